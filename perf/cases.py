@@ -154,3 +154,24 @@ def tolerance(case):
     if case["mode"] == "fft":
         return {"rel": 4e-6 if case["split"] == "tf32" else 2e-6}
     return {"rel": 1e-5}
+
+
+def exact(case, seed):
+    """The same transform in 64 bits: numpy's definition of the matrices, torch's complex128 products and transforms."""
+    shape = (case["n0"], case["n1"], case["n2"])
+    x = inputs.cube(shape, case["dist"], seed, device="cuda").to(torch.complex128)
+    nodes = _nodes(case, seed) or [None, None, None]
+    sign, spec = case["sign"], case["nodes"]
+    for a in (int(c) for c in case["axes"]):
+        if nodes[a] is None:
+            x = torch.fft.fft(x, dim=a) if sign < 0 else torch.fft.ifft(x, dim=a)
+            continue
+        k, t = np.arange(shape[a]), np.asarray(nodes[a])
+        phase = np.outer(t, k) if spec[0] == "o" else np.outer(k, t)
+        if spec[0] == "s":
+            m = np.linalg.inv(np.exp(-2j * np.pi * phase))
+        else:
+            m = np.exp(sign * 2j * np.pi * phase) / (shape[a] if sign > 0 else 1)
+        m = torch.from_numpy(m).to(x.device)
+        x = torch.movedim(torch.tensordot(m, x, dims=([1], [a])), 0, a).contiguous()
+    return x
