@@ -483,6 +483,14 @@ def main():
             algo_flops = 8.0 * nsum * P
             issued = 3.0 * algo_flops
             ach = issued / (ms * 1e-3) * 1e-12
+            if split == dft.DFT3D_SPLIT_FP16 and all(any(shape[a] % r == 0 and shape[a] // r <= 64 for r in (4, 8, 16)) for a in taxes):
+                # every axis in folded form (csrc/fold_kernel.cuh): one pass over the cube per axis, bound by HBM
+                moved = len(taxes) * 16.0 * P
+                return {"bound": "hbm", "kernel": "fold_axis_kernel", "achieved": moved / (ms * 1e-3) * 1e-9,
+                        "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": moved / (ms * 1e-3) * 1e-9 / peaks["hbm_gbs"],
+                        "traffic": (dram_bytes_per_point("fold_axis_kernel")[0] or 0.0) * P or None,
+                        "peak_source": "%s STREAM-style copy" % peak_kind, "avg_launch_ms": ms / (nlaunch - 1),
+                        "bytes": "8 B read + 8 B written per point per axis pass (the reduction over the input comes on top)"}
             if split == dft.DFT3D_SPLIT_FP16:
                 paired = max(shape[a] for a in taxes) >= 2048 and os.environ.get("DFT3D_KDFT_PAIR", "1") != "0"
                 kernel = "kdft_f16x2_axis_kernel" if paired else "kdft_f16_axis_kernel"   # CTA pairs from 2048 points up

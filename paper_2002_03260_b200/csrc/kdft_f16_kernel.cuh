@@ -54,12 +54,20 @@ struct KdftF16Shared {
   long long wait_limit;
 };
 
-// largest magnitude of a float array (grid-stride, one atomic per warp); `result` must start at zero
+// |v|, or 0 for an infinity or NaN: a line that holds one has no finite result whatever the scale, and the other lines
+// need the scale of the finite data
+__device__ __forceinline__ float finite_magnitude(float v) {
+  const float a = fabsf(v);
+  return a <= 3.402823466e38f ? a : 0.0f;
+}
+
+// largest finite magnitude of a float array (grid-stride, one atomic per warp); `result` must start at zero
 __global__ void amax_kernel(const float4* x, long long n4, unsigned int* result) {
   float m = 0.0f;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n4; i += (long long)gridDim.x * blockDim.x) {
     const float4 v = x[i];
-    m = fmaxf(fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
+    m = fmaxf(fmaxf(m, fmaxf(finite_magnitude(v.x), finite_magnitude(v.y))),
+              fmaxf(finite_magnitude(v.z), finite_magnitude(v.w)));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));

@@ -1,0 +1,94 @@
+"""The folded form of uniform KDFT axes (csrc/fold_kernel.cuh): n = R*m with R = 4, 8 or 16 and m <= 64.
+
+Bound: both operands carry 22 bits (2^-23 relative rounding each), sums and phases are fp32 (2^-24 per operation), the
+chains truncate at most 24 times: below 4e-7 per axis in the 2-norm; 1e-6 is asserted for up to three axes.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+BOUND = 1e-6
+
+
+@pytest.fixture(scope="module")
+def lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2002_03260_b200 as d
+    return d
+
+
+def _run(lib, x, **kw):
+    plan = lib.Plan(*x.shape, **kw)
+    y = plan(x)
+    torch.cuda.synchronize()
+    plan.status()
+    plan.destroy()
+    return y
+
+
+def _rel(a, b):
+    a, b = a.to(torch.complex128), b.to(torch.complex128)
+    return (torch.linalg.vector_norm((a - b).flatten()) / torch.linalg.vector_norm(b.flatten())).item()
+
+
+# every R, m from 1 to 64 with and without a remainder of the groups (of 4 and 2 points) and of the K = 16 steps, tiles that
+# are not full, batches that end inside a tile, n2 a multiple of 16 (blocked hand-over between axes 0 and 1) or not
+@pytest.mark.parametrize("shape", [(4, 4, 4), (8, 20, 12), (100, 68, 36), (256, 12, 252), (264, 8, 16), (296, 4, 24),
+                                   (512, 4, 20), (20, 504, 4), (528, 4, 32), (4, 544, 12), (36, 1008, 16), (1024, 8, 4),
+                                   (4, 12, 1008), (4, 4, 1024), (64, 64, 48)])
+@pytest.mark.parametrize("sign", [-1, +1])
+def test_folded_axes_against_the_oracle(lib, oracle, shape, sign):
+    from paper_2002_03260_b200 import inputs
+    x = inputs.cube(shape, "normal", 301, device="cuda")
+    guard = torch.full((1 << 14,), 7.0, device="cuda")
+    y = _run(lib, x, sign=sign)
+    guard2 = torch.full((1 << 14,), 7.0, device="cuda")
+    assert oracle.rel_l2(y.cpu().numpy(), oracle.dft3d(x.cpu().numpy(), sign=sign, scaled_inverse=sign > 0)) < BOUND
+    assert bool((guard == 7.0).all()) and bool((guard2 == 7.0).all())
+
+
+# the full matrix, which an axis with (uniform) nodes given keeps, in every form a plan takes
+@pytest.mark.parametrize("axes", [(0,), (1,), (2,), (0, 1), (0, 2), (1, 2), (0, 1, 2)])
+@pytest.mark.parametrize("sign,flag,limit", [(-1, "", 0), (+1, "UNSCALED_INVERSE", 0), (+1, "", 1 << 17)])
+def test_folded_axes_against_the_full_matrix(lib, axes, sign, flag, limit):
+    from paper_2002_03260_b200 import inputs
+    shape = (24, 272, 40)
+    x = inputs.cube(shape, "uniform", 302, device="cuda")
+    flags = lib.DFT3D_UNSCALED_INVERSE if flag else 0
+    if limit and 0 in axes and len(axes) == 2:
+        limit = 0                                  # such plans need a whole cube of workspace
+    uniform = [np.arange(n) / n for n in shape]
+    got = _run(lib, x, sign=sign, flags=flags, axes=axes, workspace_limit=limit)
+    want = _run(lib, x, sign=sign, flags=flags, axes=axes, nodes=uniform)
+    assert _rel(got, want) < 5e-6                  # the full matrix: 2e-6 per axis
+
+
+@pytest.mark.parametrize("scale", [2.0 ** 100, 2.0 ** 118, 2.0 ** -110])
+def test_folded_scales_at_the_ends_of_the_float_range(lib, oracle, scale):
+    """Inputs whose R-point sums would leave the float range, or that are nearly subnormal, scale like any other."""
+    from paper_2002_03260_b200 import inputs
+    shape = (4, 12, 528)
+    x = inputs.cube(shape, "normal", 303, device="cuda")
+    y = _run(lib, x, axes=(2,))
+    ys = _run(lib, x * scale, axes=(2,))
+    assert torch.equal(torch.view_as_real(ys), torch.view_as_real(y) * scale)
+    assert oracle.rel_l2(y.cpu().numpy(), oracle.dft_axis(x.cpu().numpy().astype(np.complex128), 2)) < BOUND
+
+
+def test_lines_beside_an_infinity_keep_their_values(lib):
+    """One infinite and one NaN sample: their lines are lost, the others are what they are without them."""
+    from paper_2002_03260_b200 import inputs
+    x = inputs.cube((4, 8, 528), "normal", 304, device="cuda") * 1e5
+    y = _run(lib, x, axes=(2,))
+    bad = x.clone()
+    bad[1, 3, 7] = complex(float("inf"), 0.0)
+    bad[2, 5, 9] = complex(0.0, float("nan"))
+    z = _run(lib, bad, axes=(2,))
+    lost = torch.zeros(4, 8, dtype=torch.bool, device="cuda")
+    lost[1, 3] = lost[2, 5] = True
+    assert not bool(torch.isfinite(torch.view_as_real(z[lost])).all())
+    assert _rel(z[~lost], y[~lost]) < 1e-6         # the scale may differ by a power of two, the pieces with it
