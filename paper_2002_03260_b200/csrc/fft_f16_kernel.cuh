@@ -161,6 +161,7 @@ __device__ __forceinline__ void fft_f16_axis_body(const CUtensorMap* map_data_p,
   constexpr int NL = R * R;            // length of a (sub-)line
   constexpr int kRowBytes = COLS * 8;  // STRIDED: bytes of one row of a raw stage
 
+  ptx::griddep_launch();
   if (tid == 0) {
     for (int i = 0; i < 4; ++i) {
       ptx::mbar_init(&sh.raw_full[i], 1);
@@ -190,6 +191,7 @@ __device__ __forceinline__ void fft_f16_axis_body(const CUtensorMap* map_data_p,
     ptx::prefetch_tensormap(&map_data);
     ptx::prefetch_tensormap(&map_w);
   }
+  ptx::griddep_wait();
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();

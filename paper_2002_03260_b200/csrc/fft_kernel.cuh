@@ -165,6 +165,7 @@ fft_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid_const
   constexpr int NL = R * R;            // length of a (sub-)line
   constexpr int kRowBytes = COLS * 8;  // STRIDED: bytes of one row of a raw stage
 
+  ptx::griddep_launch();
   if (tid == 0) {
     for (int i = 0; i < 4; ++i) {
       ptx::mbar_init(&sh.raw_full[i], 1);
@@ -188,6 +189,7 @@ fft_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid_const
     ptx::prefetch_tensormap(&map_data);
     ptx::prefetch_tensormap(&map_w);
   }
+  ptx::griddep_wait();
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();

@@ -256,6 +256,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
   FoldShared& sh = *reinterpret_cast<FoldShared*>(smem_tn + t_entries);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
+  ptx::griddep_launch();
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) {
       ptx::mbar_init(&sh.a_full[i], p.tasks);
@@ -276,6 +277,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
     ptx::tmem_alloc(&sh.tmem_base, 512);
     ptx::tmem_relinquish();
   }
+  ptx::griddep_wait();
   // The largest |component| of the input, at most 2^(e+1), is scaled so that the R-point sums (modulus at most R*sqrt(2)
   // times that) stay below 2^15.5.  The scale rides on the phases; data near the top of the float range are brought down
   // first so that the sums cannot overflow.

@@ -61,17 +61,50 @@ __device__ __forceinline__ float finite_magnitude(float v) {
   return a <= 3.402823466e38f ? a : 0.0f;
 }
 
-// largest finite magnitude of a float array (grid-stride, one atomic per warp); `result` must start at zero
-__global__ void amax_kernel(const float4* x, long long n4, unsigned int* result) {
+// Largest finite magnitude of a float array -> words[0]; words[1..clear] (those of the passes that follow) are set to zero.
+// Every block leaves its maximum in `scratch`, the last one to finish reduces them: no word has to be cleared before the
+// launch.  scratch[0] counts the finished blocks and wraps to zero by itself.
+constexpr int kAmaxThreads = 256, kAmaxUnroll = 4;
+__global__ void __launch_bounds__(kAmaxThreads) amax_kernel(const float4* x, long long n4, unsigned int* words, int clear,
+                                                            unsigned int* scratch) {
+  __shared__ unsigned int part[kAmaxThreads / 32];
+  __shared__ bool last;
+  ptx::griddep_launch();
+  ptx::griddep_wait();
   float m = 0.0f;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n4; i += (long long)gridDim.x * blockDim.x) {
-    const float4 v = x[i];
-    m = fmaxf(fmaxf(m, fmaxf(finite_magnitude(v.x), finite_magnitude(v.y))),
-              fmaxf(finite_magnitude(v.z), finite_magnitude(v.w)));
-  }
+  const long long step = (long long)gridDim.x * kAmaxThreads;
+  for (long long i = blockIdx.x * (long long)kAmaxThreads + threadIdx.x; i < n4; i += step * kAmaxUnroll) {
+    float4 v[kAmaxUnroll];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0 && m > 0.0f) atomicMax(result, __float_as_uint(m));
+    for (int u = 0; u < kAmaxUnroll; ++u) v[u] = i + u * step < n4 ? x[i + u * step] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < kAmaxUnroll; ++u)
+      m = fmaxf(fmaxf(m, fmaxf(finite_magnitude(v[u].x), finite_magnitude(v[u].y))),
+                fmaxf(finite_magnitude(v[u].z), finite_magnitude(v[u].w)));
+  }
+  // non-negative floats compare like their bits
+  unsigned int r = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = r;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kAmaxThreads / 32; ++w) r = max(r, part[w]);
+    scratch[1 + blockIdx.x] = r;
+    __threadfence();
+    last = atomicInc(scratch, gridDim.x - 1) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  r = 0;
+  for (unsigned int b = threadIdx.x; b < gridDim.x; b += kAmaxThreads) r = max(r, __ldcg(scratch + 1 + b));
+  r = __reduce_max_sync(0xffffffffu, r);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = r;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kAmaxThreads / 32; ++w) r = max(r, part[w]);
+    words[0] = r;
+    for (int w = 1; w <= clear; ++w) words[w] = 0;
+  }
 }
 
 // single-thread wait (producer, MMA issuer)
@@ -104,6 +137,7 @@ kdft_f16_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid_
   const int warp = tid >> 5;
   const int lane = tid & 31;
 
+  ptx::griddep_launch();
   if (tid == 0) {
     for (int i = 0; i < kStagesB; ++i) { ptx::mbar_init(&sh.b_full[i], 1); ptx::mbar_init(&sh.b_empty[i], 1); }
     for (int i = 0; i < kF16HalvesA; ++i) { ptx::mbar_init(&sh.a_full[i], 1); ptx::mbar_init(&sh.a_empty[i], 4); }
@@ -122,6 +156,7 @@ kdft_f16_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid_
     ptx::prefetch_tensormap(&map_data);
     ptx::prefetch_tensormap(&map_w);
   }
+  ptx::griddep_wait();
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();

@@ -149,6 +149,7 @@ kdft_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid_cons
   const int warp = tid >> 5;
   const int lane = tid & 31;
 
+  ptx::griddep_launch();
   if (tid == 0) {
     for (int i = 0; i < kStagesB; ++i) { ptx::mbar_init(&sh.b_full[i], 1); ptx::mbar_init(&sh.b_empty[i], 1); }
     for (int i = 0; i < kStagesA; ++i) { ptx::mbar_init(&sh.a_full[i], 1); ptx::mbar_init(&sh.a_empty[i], 4); }
@@ -167,6 +168,7 @@ kdft_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid_cons
     ptx::prefetch_tensormap(&map_data);
     ptx::prefetch_tensormap(&map_w);
   }
+  ptx::griddep_wait();
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();

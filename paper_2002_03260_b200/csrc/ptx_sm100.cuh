@@ -42,6 +42,14 @@ __device__ __forceinline__ void setmaxnreg_dec() {
 #endif
 }
 
+// ---------------------------------------------------------------- dependent launches
+// A kernel launched with the programmatic attribute may start while its predecessor in the stream still runs: everything
+// that touches memory the predecessor writes or reads comes after griddep_wait (which waits until the predecessor has
+// finished and its writes are visible).  griddep_launch lets the successor's blocks start as soon as there is room.
+// Both do nothing in ordinary launches.
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------------- mbarrier
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
