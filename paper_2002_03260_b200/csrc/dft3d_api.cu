@@ -172,9 +172,11 @@ struct KdftAxis {
   float out_mul = 1.0f;   // fp16 pieces: 2^-10, times 1/n for a scaled inverse
   // uniform grid, n = fold_r * m: the matrix in folded form (fold_kernel.cuh); 0 = not folded
   int fold_r = 0;
+  bool fold_t32 = false;         // with TF32 pieces
   uint8_t* d_fold_w = nullptr;   // the m-point table as it lies in shared memory
   float4* d_fold_tw = nullptr;   // [fold_r][mp / 2] phases of pairs of points
   unsigned fold_w_bytes = 0;
+  float fold_pre = 1.0f, fold_scale = 1.0f;   // TF32 pieces: factors before the R-point sums and on the phases
 };
 
 struct FftAxis {
@@ -259,12 +261,12 @@ dft3d::WaitControl wait_control(const dft3d_plan_s* p) {
   return wc;
 }
 
-// Folded KDFT axes (fold_kernel.cuh): the number R of residue classes, n = R*m with m <= 64 so that the table fits
-// shared memory; 0 = the axis keeps the full matrix.  The smallest R that does it: the product then takes the most of
-// the work, and a tile holds the most neighbouring lines (128/R).
-int fold_radix(long long n) {
+// Folded axes (fold_kernel.cuh): the number R of residue classes, n = R*m with m <= 64 (fp16 pieces) or 32 (TF32 pieces, whose
+// operands are twice as large), so that the table and two operand buffers fit shared memory; 0 = the axis keeps its
+// other form.  The smallest R that does it: a tile then holds the most neighbouring lines (128/R).
+int fold_radix(long long n, bool f16) {
   for (int r = 4; r <= 16; r *= 2)
-    if (n % r == 0 && n / r <= 64) return r;
+    if (n % r == 0 && n / r <= (f16 ? 64 : 32)) return r;
   return 0;
 }
 constexpr size_t kFoldSmemMax = dft3d::fold_smem_bytes(64 * 1024, 2, 1024);
@@ -292,21 +294,15 @@ int set_kernel_attributes(int device) {
   DFT3D_CUDA(cudaFuncSetAttribute(dft3d::fft_axis_kernel<MODE, R, RX, COLS, NB2, SO>,                          \
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(dft3d::fft_smem_bytes(R, NB2))))
   DFT3D_FFT_ATTR(dft3d::FFT_CONTIG, 32, 1, 16, 2, 0);
-  DFT3D_FFT_ATTR(dft3d::FFT_CONTIG, 16, 1, 16, 2, 0);
   DFT3D_FFT_ATTR(dft3d::FFT_CONTIG, 32, 2, 16, 2, 0);
-  DFT3D_FFT_ATTR(dft3d::FFT_CONTIG, 16, 2, 16, 2, 0);
   DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 32, 1, 16, 1, 0);
   DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 32, 1, 8, 2, 0);
-  DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 16, 1, 16, 2, 0);
   DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 32, 2, 8, 1, 0);
-  DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 16, 2, 16, 2, 0);
   DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 32, 1, 16, 1, 1);
   DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 32, 1, 8, 1, 0);
   DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 32, 1, 8, 1, 1);
   DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 32, 1, 8, 2, 1);
-  DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 16, 1, 16, 2, 1);
   DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 32, 2, 8, 1, 1);
-  DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 16, 2, 16, 2, 1);
 #undef DFT3D_FFT_ATTR
 #define DFT3D_FFT16_ATTR(MODE, R, RX, COLS, SO)                                                   \
   DFT3D_CUDA(cudaFuncSetAttribute(dft3d::fft_f16_axis_kernel<MODE, R, RX, COLS, SO>,              \
@@ -329,14 +325,17 @@ int set_kernel_attributes(int device) {
   DFT3D_FFT16_ATTR(dft3d::FFT_STRIDED, 32, 4, 4, 0);
   DFT3D_FFT16_ATTR(dft3d::FFT_STRIDED, 32, 4, 4, 1);
 #undef DFT3D_FFT16_ATTR
-#define DFT3D_FOLD_ATTR(R)                                                                                       \
-  DFT3D_CUDA(cudaFuncSetAttribute(dft3d::fold_axis_kernel<dft3d::KDFT_CONTIG, R>,                                  \
+#define DFT3D_FOLD_ATTR(R, T32)                                                                                  \
+  DFT3D_CUDA(cudaFuncSetAttribute(dft3d::fold_axis_kernel<dft3d::KDFT_CONTIG, R, T32>,                             \
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(kFoldSmemMax)));               \
-  DFT3D_CUDA(cudaFuncSetAttribute(dft3d::fold_axis_kernel<dft3d::KDFT_STRIDED, R>,                                 \
+  DFT3D_CUDA(cudaFuncSetAttribute(dft3d::fold_axis_kernel<dft3d::KDFT_STRIDED, R, T32>,                            \
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(kFoldSmemMax)))
-  DFT3D_FOLD_ATTR(4);
-  DFT3D_FOLD_ATTR(8);
-  DFT3D_FOLD_ATTR(16);
+  DFT3D_FOLD_ATTR(4, false);
+  DFT3D_FOLD_ATTR(8, false);
+  DFT3D_FOLD_ATTR(16, false);
+  DFT3D_FOLD_ATTR(4, true);
+  DFT3D_FOLD_ATTR(8, true);
+  DFT3D_FOLD_ATTR(16, true);
 #undef DFT3D_FOLD_ATTR
   DFT3D_CUDA(cudaFuncSetAttribute(dft3d::fft_f16_fused_kernel<32, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   int(dft3d::fft16_smem_bytes(32, 1))));
@@ -346,33 +345,41 @@ int set_kernel_attributes(int device) {
   return DFT3D_OK;
 }
 
-// Tables of a folded axis: the real form of the m-point matrix in two fp16 pieces (1024*W = hi + 2^-11*lo'), laid out and
-// swizzled as the kernel's shared memory holds it, and the phases exp(s*2*pi*i*i*q/n) in rows of mp >= m.
-int build_fold_axis(dft3d_plan_s* p, KdftAxis& ax, int r, double scale) {
+// Tables of a folded axis: the real form of the m-point matrix in two pieces (fp16: 1024*W = hi + 2^-11*lo'; TF32: W = hi + lo),
+// laid out and swizzled as the kernel's shared memory holds it, and the phases exp(s*2*pi*i*i*q/n) in rows of mp >= m.
+int build_fold_axis(dft3d_plan_s* p, KdftAxis& ax, int r, bool t32, double scale) {
   const int m = int(ax.n) / r, B = dft3d::fold_group(r), mp = (m + B - 1) / B * B;
-  const int np = (2 * m + 15) / 16 * 16, panels = (2 * m + 63) / 64;
+  const int words = t32 ? 32 : 64;                     // operand words per row of 128 bytes
+  const int np = (2 * m + 15) / 16 * 16, panels = (2 * m + words - 1) / words;
   std::vector<double> M;
-  std::vector<__half> W;
+  std::vector<uint8_t> W;
   std::vector<float> tw;
   try {
     M.resize(size_t(2) * m * m);
-    W.assign(size_t(panels) * 2 * np * 64, __float2half_rn(0.0f));
+    W.assign(size_t(panels) * 2 * np * 128, 0);
     tw.assign(size_t(2) * r * mp, 0.0f);
   } catch (const std::bad_alloc&) {
     return fail(DFT3D_ERR_ALLOC, "host allocation of a folded table failed");
   }
-  dft3d::gen::axis_matrix(m, p->sign, 1024.0, nullptr, false, M.data());
+  dft3d::gen::axis_matrix(m, p->sign, t32 ? 1.0 : 1024.0, nullptr, false, M.data());
   for (int k = 0; k < m; ++k)
     for (int j = 0; j < m; ++j)
       for (int e = 0; e < 4; ++e) {                       // (row, column) = (2k + e/2, 2j + e%2)
         const double re = M[2 * (size_t(k) * m + j)], im = M[2 * (size_t(k) * m + j) + 1];
         const double v = e == 0 || e == 3 ? re : (e == 1 ? -im : im);
-        const double hi = dft3d::gen::round_to_fp16(v);
-        const double lo = dft3d::gen::round_to_fp16((v - hi) * 2048.0);
-        const int col = 2 * j + e % 2, pn = col / 64, h = col % 64;
+        const int col = 2 * j + e % 2, pn = col / words, h = col % words, per_chunk = words / 8;
         for (int pc = 0; pc < 2; ++pc) {
           const int row = pc * np + 2 * k + e / 2;
-          W[((size_t(pn) * 2 * np + row) * 64) + ((h / 8) ^ (row & 7)) * 8 + h % 8] = __float2half_rn(float(pc ? lo : hi));
+          uint8_t* at = &W[(size_t(pn) * 2 * np + row) * 128 + ((h / per_chunk) ^ (row & 7)) * 16 + h % per_chunk * (128 / words)];
+          if (!t32) {
+            const double hi = dft3d::gen::round_to_fp16(v);
+            const __half x = __float2half_rn(float(pc ? dft3d::gen::round_to_fp16((v - hi) * 2048.0) : hi));
+            memcpy(at, &x, sizeof(x));
+          } else {
+            const float hi = dft3d::gen::round_to_tf32(v);
+            const float x = pc ? dft3d::gen::round_to_tf32(v - double(hi)) : hi;
+            memcpy(at, &x, sizeof(x));
+          }
         }
       }
   for (int q = 0; q < r; ++q)
@@ -384,10 +391,17 @@ int build_fold_axis(dft3d_plan_s* p, KdftAxis& ax, int r, double scale) {
       pair[2 + i % 2] = float(im);
     }
   ax.fold_r = r;
-  ax.fold_w_bytes = unsigned(W.size() * sizeof(__half));
-  ax.out_mul = float(scale / 1024.0);
-  DFT3D_CUDA(cudaMalloc(&ax.d_fold_w, W.size() * sizeof(__half)));
-  DFT3D_CUDA(cudaMemcpy(ax.d_fold_w, W.data(), W.size() * sizeof(__half), cudaMemcpyHostToDevice));
+  ax.fold_w_bytes = unsigned(W.size());
+  ax.fold_t32 = t32;
+  if (!t32) {
+    ax.out_mul = float(scale / 1024.0);
+  } else if (scale != 1.0) {
+    // TF32 pieces carry no scale that keeps large data in range, so the 1/n of a scaled inverse is taken before the sums
+    ax.fold_pre = 1.0f / float(r);
+    ax.fold_scale = 1.0f / float(m);
+  }
+  DFT3D_CUDA(cudaMalloc(&ax.d_fold_w, W.size()));
+  DFT3D_CUDA(cudaMemcpy(ax.d_fold_w, W.data(), W.size(), cudaMemcpyHostToDevice));
   DFT3D_CUDA(cudaMalloc(&ax.d_fold_tw, tw.size() * sizeof(float)));
   DFT3D_CUDA(cudaMemcpy(ax.d_fold_tw, tw.data(), tw.size() * sizeof(float), cudaMemcpyHostToDevice));
   return DFT3D_OK;
@@ -400,8 +414,9 @@ int build_kdft_axis(dft3d_plan_s* p, int a, const double* nodes) {
   ax.bn = int(2 * n < 256 ? (2 * n + 15) / 16 * 16 : 256);   // MMA N: a multiple of 16, rows beyond 2n are zero-filled
   const bool scaled = (p->sign > 0) && !(p->flags & DFT3D_UNSCALED_INVERSE);
   const double scale = scaled ? 1.0 / double(n) : 1.0;
-  // fp16 pieces on a uniform grid: the folded form where the length has one (line numbers are 32-bit there)
-  if (p->f16 && !nodes && fold_radix(n) && points(p) / n < (1ll << 31)) return build_fold_axis(p, ax, fold_radix(n), scale);
+  // uniform grid: the folded form where the length has one (line numbers are 32-bit there)
+  const int fold = fold_radix(n, p->f16);
+  if (!nodes && fold && points(p) / n < (1ll << 31)) return build_fold_axis(p, ax, fold, !p->f16, scale);
   std::vector<double> M;
   std::vector<float> W;
   try {
@@ -641,9 +656,10 @@ int launch_kdft_contig(dft3d_plan_s* p, int a, const float* in, float* out, long
   return DFT3D_OK;
 }
 
-// blocked: axis 0 writes, axis 1 reads the blocked order of fold_place
+// blocked: axis 0 writes, axis 1 reads the blocked order of fold_place, in blocks of that many columns (0 = natural order)
+// n2_sub != 0: only the slice [n2_off, n2_off + n2_sub) of the last axis (axes 0 and 1, one of the two sides blocked)
 int launch_fold(dft3d_plan_s* p, int a, const float* in, float* out, long long lines, long long C, cudaStream_t stream,
-                int chain_pos, bool blocked) {
+                int chain_pos, int blocked, long long n2_off = 0, long long n2_sub = 0) {
   const KdftAxis& ax = p->kax[a];
   const int r = ax.fold_r, m = int(ax.n) / r, B = dft3d::fold_group(r);
   const int H = dft3d::fold_tiles(a != 2, r), L = dft3d::fold_lines(a != 2, r);
@@ -658,25 +674,30 @@ int launch_fold(dft3d_plan_s* p, int a, const float* in, float* out, long long l
   fp.groups = unsigned((m + B - 1) / B);
   fp.mp = int(fp.groups) * B;
   fp.np = (2 * m + 15) / 16 * 16;
-  fp.ks = (2 * m + 15) / 16;
-  fp.panels = (2 * m + 63) / 64;
+  fp.ks = ax.fold_t32 ? (2 * m + 7) / 8 : (2 * m + 15) / 16;
+  fp.panels = (fp.ks + 3) / 4;
+  fp.pre = ax.fold_pre;
+  fp.in_scale = ax.fold_scale;
   fp.w_bytes = ax.fold_w_bytes;
   fp.groups_magic = ((1u << 24) + fp.groups - 1) / fp.groups;
-  fp.lines = unsigned(lines);
-  fp.C = unsigned(C);
+  fp.lines = unsigned(n2_sub ? lines / p->n[2] * n2_sub : lines);
+  fp.C = unsigned(n2_sub ? n2_sub : C);
+  fp.off = unsigned(n2_off);
+  fp.pitch = size_t(n2_sub && a == 0 ? p->n[2] : ax.n * C);   // a slice of axis 0: one stretch of columns per i1
+  fp.step = size_t(C);
   fp.units = unsigned((lines + L - 1) / L);
   fp.tasks = (unsigned(L) * fp.groups + 31) / 32;
   // see the kernel's loop over tasks: a unit of two tiles fills both buffers, a unit of one tile every other one
   const unsigned warps = H == 2 ? fp.tasks : 2 * fp.tasks;
   fp.split_warps = int(warps < unsigned(dft3d::kFoldSplitWarps) ? warps : unsigned(dft3d::kFoldSplitWarps));
-  fp.in_blocked = blocked && a == 1;
+  fp.in_blocked = a == 1 ? blocked : 0;
   // Rows a MiB and more apart: the pass is bound by address translations, and prefetches add to them (512 x 1024 x 1024, axis 0
   // in natural order: 2.26 ms without, 2.73 ms with); closer rows gain (axis 1: 2.15 -> 1.82 ms)
   fp.prefetch = a == 2 || C * 8 < (1 << 20);
-  fp.out_blocked = blocked && a == 0;
+  fp.out_blocked = a == 0 ? blocked : 0;
   fp.n0 = unsigned(p->n[0]);
   fp.n1 = unsigned(p->n[1]);
-  fp.n2 = unsigned(p->n[2]);
+  fp.n2 = unsigned(n2_sub ? n2_sub : p->n[2]);
   fp.out_mul = ax.out_mul;
   fp.amax_in = p->d_amax + chain_pos;
   fp.amax_out = p->d_amax + chain_pos + 1;
@@ -685,8 +706,11 @@ int launch_fold(dft3d_plan_s* p, int a, const float* in, float* out, long long l
   const int grid = int(fp.units < unsigned(p->sm_count) ? fp.units : unsigned(p->sm_count));
   const size_t smem = dft3d::fold_smem_bytes(fp.w_bytes, fp.panels, r * fp.mp);
   const float sign = float(p->sign);
-#define DFT3D_FOLD_LAUNCH(MODE, R)                                                                    \
-  DFT3D_CUDA(launch_overlapped(p, dft3d::fold_axis_kernel<MODE, R>, grid, dft3d::kFoldThreads, smem, stream, fp, sign))
+#define DFT3D_FOLD_LAUNCH(MODE, R)                                                                                       \
+  DFT3D_CUDA(ax.fold_t32 ? launch_overlapped(p, dft3d::fold_axis_kernel<MODE, R, true>, grid, dft3d::kFoldThreads, smem,   \
+                                             stream, fp, sign)                                                            \
+                         : launch_overlapped(p, dft3d::fold_axis_kernel<MODE, R, false>, grid, dft3d::kFoldThreads, smem,  \
+                                             stream, fp, sign))
   if (a == 2) {
     if (r == 4) { DFT3D_FOLD_LAUNCH(dft3d::KDFT_CONTIG, 4); }
     else if (r == 8) { DFT3D_FOLD_LAUNCH(dft3d::KDFT_CONTIG, 8); }
@@ -708,7 +732,7 @@ bool fold_blocked(const dft3d_plan_s* p) {
 }
 
 int kdft_axis_pass(dft3d_plan_s* p, int axis, const float* in, float* out, long long planes, cudaStream_t stream,
-                   int chain_pos, bool blocked = false) {
+                   int chain_pos, int blocked = 0) {
   // `planes` n0-planes starting at in/out (axis 0 always takes the whole cube)
   const long long n1 = p->n[1], n2 = p->n[2];
   if (p->kax[axis].fold_r) {
@@ -770,6 +794,14 @@ int build_fft_axis(dft3d_plan_s* p, int a, const int split[2]) {
   ax.RX = RX;
   ax.cols = (R == 32 && RX == 4) ? 4 : ((R == 32 && RX == 2) ? 8 : 16);   // a 128 KB stage holds all n rows of `cols` lines
                                                                            // (fft_axis_pass may pick 8 for R = 32, RX = 1)
+  // One product in folded form, with TF32 pieces, instead of two: always where the plan has TF32 pieces, and on 512-point axes
+  // of plans that leave the pieces open (512^3, microseconds per pass, this against fp16 pieces: axis 0 491 / 577,
+  // axis 1 415 / 565, axis 2 394 / 428; no scaling and no larger error).  256 points: 58 to 63 against 59 to 69 at 256^3, which
+  // is too little to give up the arithmetic that the launch over axes 1 and 2 shares.
+  if (fold_radix(n, false) && (!p->f16 || (n == 512 && !(p->flags & DFT3D_SPLIT_FP16)))) {
+    p->kax[a].n = n;
+    return build_fold_axis(p, p->kax[a], fold_radix(n, false), true, scaled ? 1.0 / double(n) : 1.0);
+  }
   const int K = 2 * R, NB = 2 * R, panels = K / 32;
   if (p->f16) {
     // fp16 pieces: 1024 * F_R (real form), rows of 64 halves (zero-padded for R = 16), [hi piece; lo piece]; the twiddle
@@ -884,7 +916,7 @@ int fft_cols_for(const dft3d_plan_s* p, int axis, int layout) {
 // Blocked intermediate, fp16-piece kernel with direct stores: how many neighbouring rows i1 share the 128-byte lines
 // of a block (see FftParams::blk_pair).  1 when the stages are 128 bytes wide anyway, or where the two passes differ.
 int fft_blk_pair(const dft3d_plan_s* p) {
-  if (!p->f16 || p->knobs.fft_no_pair) return 1;
+  if (!p->f16 || p->knobs.fft_no_pair || p->kax[0].fold_r || p->kax[1].fold_r) return 1;
   if (p->knobs.fft_stage_out_blocked > 0) return 1;
   const int colsA = fft_cols_for(p, 0, FFT_OUT_BLOCKED), cols1 = fft_cols_for(p, 1, FFT_IN_BLOCKED);
   if (cols1 != colsA) return 1;
@@ -916,6 +948,11 @@ int fft_axis_pass(dft3d_plan_s* p, int axis, const float* in, float* out, cudaSt
                   int layout = FFT_NATURAL, long long n2_off = 0, long long n2_sub = 0, long long map_rows = 0,
                   FftCapture* capture = nullptr, const FftView* view = nullptr) {
   const FftAxis& ax = p->fax[axis];
+  if (p->kax[axis].fold_r) {     // see build_fft_axis
+    const long long C = axis == 0 ? p->n[1] * p->n[2] : (axis == 1 ? p->n[2] : 1);
+    return launch_fold(p, axis, in, out, points(p) / ax.n, C, stream, 0,
+                       layout == FFT_NATURAL ? 0 : fft_cols_for(p, 0, FFT_OUT_BLOCKED), n2_off, n2_sub);
+  }
   const int R = ax.R, RX = ax.RX, N = int(ax.n), Lg = 128 / (R * RX);
   const int cols = view ? view->cols : fft_cols_for(p, axis, layout);
   dft3d::FftParams fp;
@@ -1087,7 +1124,7 @@ int fft_axis_pass(dft3d_plan_s* p, int axis, const float* in, float* out, cudaSt
     DFT3D_CUDA(cudaGetLastError());
     return DFT3D_OK;
   }
-  int nb2 = (axis == 2 || R == 16 || (R == 32 && RX == 1 && cols == 8)) ? 2 : 1;
+  int nb2 = (axis == 2 || (RX == 1 && cols == 8)) ? 2 : 1;   // R = 32: the shorter lengths run folded
   if (axis != 2 && R == 32 && RX == 1 && cols == 8) {
     // 8-line stages: two stage-2 operand buffers and one raw stage (best with direct stores), or one operand
     // buffer and two raw stages (best when the results return through the raw stage, which then stays busy longer)
@@ -1103,23 +1140,17 @@ int fft_axis_pass(dft3d_plan_s* p, int axis, const float* in, float* out, cudaSt
                                stream, map_data, ax.map_w, map_out, fp))
   if (axis == 2) {
     if (R == 32 && RX == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_CONTIG, 32, 1, 16, 2, 0); }
-    else if (R == 16 && RX == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_CONTIG, 16, 1, 16, 2, 0); }
-    else if (R == 32) { DFT3D_FFT_LAUNCH(dft3d::FFT_CONTIG, 32, 2, 16, 2, 0); }
-    else { DFT3D_FFT_LAUNCH(dft3d::FFT_CONTIG, 16, 2, 16, 2, 0); }
+    else { DFT3D_FFT_LAUNCH(dft3d::FFT_CONTIG, 32, 2, 16, 2, 0); }
   } else if (!stage_out) {
     if (R == 32 && RX == 1 && cols == 16) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 1, 16, 1, 0); }
     else if (R == 32 && RX == 1 && nb2 == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 1, 8, 1, 0); }
     else if (R == 32 && RX == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 1, 8, 2, 0); }
-    else if (R == 16 && RX == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 16, 1, 16, 2, 0); }
-    else if (R == 32) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 2, 8, 1, 0); }
-    else { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 16, 2, 16, 2, 0); }
+    else { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 2, 8, 1, 0); }
   } else {
     if (R == 32 && RX == 1 && cols == 16) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 1, 16, 1, 1); }
     else if (R == 32 && RX == 1 && nb2 == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 1, 8, 1, 1); }
     else if (R == 32 && RX == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 1, 8, 2, 1); }
-    else if (R == 16 && RX == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 16, 1, 16, 2, 1); }
-    else if (R == 32) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 2, 8, 1, 1); }
-    else { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 16, 2, 16, 2, 1); }
+    else { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 2, 8, 1, 1); }
   }
 #undef DFT3D_FFT_LAUNCH
   DFT3D_CUDA(cudaGetLastError());
@@ -1610,7 +1641,7 @@ int dft3d_execute(dft3d_plan_t p, const void* in, void* out, void* cuda_stream) 
     // still an upper bound for its own data)
     if (axes == 7u) {
       // axis 0: in -> out; then per group of n0-planes: axis 1 out -> workspace, axis 2 workspace -> out
-      const bool blocked = fold_blocked(p);
+      const int blocked = fold_blocked(p) ? 16 : 0;
       if ((rc = kdft_axis_pass(p, 0, fin, fout, p->n[0], stream, 0, blocked)) != DFT3D_OK) return rc;
       for (long long a = 0; a < p->n[0]; a += g) {
         float* slab = fout + a * plane_floats;

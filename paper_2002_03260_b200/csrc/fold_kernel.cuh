@@ -37,19 +37,22 @@ namespace dft3d {
 struct FoldParams {
   const float2* in;
   float2* out;
-  const uint8_t* w_image;   // table as it lies in shared memory: [panel of 64 halves][hi rows, lo' rows][128 B], swizzled
+  const uint8_t* w_image;   // table as it lies in shared memory: [panel of 128 bytes][hi rows, lo rows][128 B], swizzled
   const float4* tw;         // [R][mp/2] phases exp(+-2*pi*i*i*q/N) of i, i+1: (re, re', im, im'), zero beyond m
   int n, m, mp;             // N, m, m rounded up to whole groups
   int np;                   // MMA N of one piece: 2m rounded up to 16
-  int ks;                   // K = 16 steps
-  int panels;               // panels of 64 halves
+  int ks;                   // MMA steps along the contraction: 32 bytes, K = 16 halves or 8 TF32 words
+  int panels;               // panels of 128 bytes
   unsigned w_bytes;
   unsigned groups;          // groups of B consecutive i per line
   unsigned groups_magic;    // ceil(2^24 / groups)
-  unsigned lines, C;        // C: columns per batch (STRIDED)
+  unsigned lines;
+  unsigned C, off;          // STRIDED, natural order: line l starts at (l / C) * pitch + off + l % C, its points are `step` apart
+  size_t pitch, step;
   int prefetch;             // L2 prefetch of later units
-  int in_blocked, out_blocked;   // layouts of the intermediate between axes 0 and 1, see fold_place
-  unsigned n0, n1, n2;      // the cube (blocked layouts only)
+  float pre, in_scale;      // TF32 pieces: factors before the R-point sums and on the phases (fp16: from amax_in)
+  int in_blocked, out_blocked;   // columns per block, 0 = natural order: layouts of the intermediate between axes 0 and 1, see fold_place
+  unsigned n0, n1, n2;      // the cube or the slice of its last axis (blocked layouts only)
   unsigned units;           // groups of fold_lines lines
   unsigned tasks;           // warp-sized shares of a unit's loads and sums
   int split_warps;          // warps that take them
@@ -77,7 +80,7 @@ __host__ __device__ constexpr int fold_group(int R) { return R == 16 ? 2 : 4; }
 // from DRAM twice: 1.8 instead of 1.07 GB at 128 x 1024 x 1024, 652 us.)
 __host__ __device__ constexpr int fold_tiles(bool strided, int R) { return strided && R == 16 ? 2 : 1; }
 __host__ __device__ constexpr int fold_lines(bool strided, int R) { return 128 / R * fold_tiles(strided, R); }
-constexpr int kFoldPanelBytes = 128 * 128;      // 128 lanes x 64 halves
+constexpr int kFoldPanelBytes = 128 * 128;      // 128 lanes x 128 bytes
 __host__ __device__ constexpr size_t fold_smem_bytes(unsigned w_bytes, int panels, int tw_entries) {
   return size_t(w_bytes) + size_t(4) * panels * kFoldPanelBytes + size_t(tw_entries) * 12 + sizeof(FoldShared) + 1024;
 }
@@ -176,6 +179,19 @@ __device__ __forceinline__ void split_half2_scaled(C2 x, uint32_t& hi0, uint32_t
   lo1 = *reinterpret_cast<const uint32_t*>(&l1);
 }
 
+// Two complex numbers -> TF32 pieces (re, im, re', im'): hi is the raw word (the tensor core ignores the low 13 bits of the
+// mantissa), lo the remainder rounded to TF32.
+__device__ __forceinline__ void split_tf32(C2 x, uint32_t (&hi)[4], uint32_t (&lo)[4]) {
+  float v[4];
+  unpack2(x.re, v[0], v[2]);
+  unpack2(x.im, v[1], v[3]);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    hi[i] = __float_as_uint(v[i]);
+    lo[i] = (__float_as_uint(v[i] - __uint_as_float(hi[i] & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
+  }
+}
+
 // Loads of the data, and explicit shared-memory accesses.  The 8-byte form takes whole lines per warp; of the 16-byte form a
 // warp's lanes may be 32 bytes apart, and the second load finds the other halves of the sectors in L1 (512-point lines:
 // 582 us with, 620 us without).
@@ -201,7 +217,7 @@ __device__ __forceinline__ void sts_128(uint32_t addr, uint32_t a, uint32_t b, u
 }
 
 // Where line l starts and how far apart its points are, in complex numbers.  Natural order: [batch][j][C].  Blocked order,
-// between the passes over axis 0 and axis 1 of one transform: [n2 / 16][i1][k0][16 columns], in which the axis-0 pass
+// between the passes over axis 0 and axis 1 of one transform: [n2 / 16][i1][k0][16 columns] (eight where one of the two axes has no folded form), in which the axis-0 pass
 // writes contiguous blocks (its rows are n1*n2 points apart in natural order, and writing such rows piecewise is slow)
 // and the axis-1 pass reads whole 128-byte lines.
 struct LinePlace {
@@ -209,15 +225,15 @@ struct LinePlace {
 };
 __device__ __forceinline__ LinePlace fold_place(const FoldParams& p, unsigned l, bool in_blocked, bool out_blocked) {
   if (in_blocked) {            // axis 1: l = k0 * n2 + i2
-    const unsigned b = l / p.C, c = l - b * p.C;
-    return {(size_t(c >> 4) * p.n1 * p.n0 + b) * 16 + (c & 15), size_t(p.n0) * 16};
+    const unsigned b = l / p.C, c = l - b * p.C, w = unsigned(p.in_blocked), t = w == 16 ? c >> 4 : c / w;
+    return {(size_t(t) * p.n1 * p.n0 + b) * w + (c - t * w), size_t(p.n0) * w};
   }
   if (out_blocked) {           // axis 0: l = i1 * n2 + i2
-    const unsigned i1 = l / p.n2, i2 = l - i1 * p.n2;
-    return {(size_t(i2 >> 4) * p.n1 + i1) * p.n0 * 16 + (i2 & 15), 16};
+    const unsigned i1 = l / p.n2, i2 = l - i1 * p.n2, w = unsigned(p.out_blocked), t = w == 16 ? i2 >> 4 : i2 / w;
+    return {(size_t(t) * p.n1 + i1) * p.n0 * w + (i2 - t * w), w};
   }
   const unsigned b = l / p.C, c = l - b * p.C;
-  return {size_t(b) * p.n * p.C + c, p.C};
+  return {size_t(b) * p.pitch + p.off + c, p.step};
 }
 
 #define FOLD_WAIT(bar, parity, code)                                                   \
@@ -233,7 +249,8 @@ __device__ __forceinline__ LinePlace fold_place(const FoldParams& p, unsigned l,
     goto role_done;                                                                                       \
   }
 
-template <int MODE, int R>
+// T32: TF32 pieces instead of fp16 ones (no scaling; twice the bytes per operand, so m <= 32)
+template <int MODE, int R, bool T32>
 __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldParams p, const float sign) {
   constexpr int H = fold_tiles(MODE == KDFT_STRIDED, R);   // tiles per unit
   constexpr int Q = R / H;          // residue classes per tile
@@ -282,7 +299,10 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
   // times that) stay below 2^15.5.  The scale rides on the phases; data near the top of the float range are brought down
   // first so that the sums cannot overflow.
   float in_scale = 1.0f, out_mul2 = 1.0f, pre = 1.0f;
-  {
+  if (T32) {
+    in_scale = p.in_scale;
+    pre = p.pre;
+  } else {
     const float a = __uint_as_float(*p.amax_in);
     if (a > 0.0f && a < 3.0e38f) {
       constexpr int kTop = 14 - kLog2R;
@@ -298,7 +318,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
     smem_t[i] = make_float4(t.x * in_scale, t.y * in_scale, t.z * in_scale, t.w * in_scale);
     smem_tn[i] = make_float2(-t.z * in_scale, -t.w * in_scale);
   }
-  if (2 * p.mp < 16 * p.ks) {   // columns of the contraction that no group writes
+  if (2 * p.mp < (T32 ? 8 : 16) * p.ks) {   // columns of the contraction that no group writes
     uint4* z = reinterpret_cast<uint4*>(smem_a);
     for (uint32_t i = tid; i < 4 * piece_bytes / 16; i += kFoldThreads) z[i] = make_uint4(0, 0, 0, 0);
     ptx::fence_proxy_async_smem();
@@ -316,8 +336,8 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
     ptx::setmaxnreg_dec<40>();
     if (warp == 0 && lane == 0) {
       // ------------------------------------------------------------ MMA issuer
-      const uint32_t idesc = ptx::make_idesc_f16(128, p.np);
-      const uint32_t idesc_wide = ptx::make_idesc_f16(128, 2 * p.np);
+      const uint32_t idesc = T32 ? ptx::make_idesc_tf32(128, p.np) : ptx::make_idesc_f16(128, p.np);
+      const uint32_t idesc_wide = T32 ? ptx::make_idesc_tf32(128, 2 * p.np) : ptx::make_idesc_f16(128, 2 * p.np);
       const uint64_t w0 = ptx::make_kmajor_sw128_desc(ptx::smem_u32(smem_w));
       const uint64_t a0 = ptx::make_kmajor_sw128_desc(ptx::smem_u32(smem_a));
       const uint32_t w_panel = uint32_t(2 * p.np * 128) >> 4;     // in descriptor address units
@@ -332,8 +352,13 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
         for (int s = 0; s < p.ks; ++s) {
           const uint32_t a_off = uint32_t(s >> 2) * (kFoldPanelBytes >> 4) + (s & 3) * 2;
           const uint64_t wd = w0 + uint32_t(s >> 2) * w_panel + (s & 3) * 2;
-          ptx::mma_f16_ss(d, ah + a_off, wd, idesc_wide, s != 0);
-          ptx::mma_f16_ss(d + p.np, al + a_off, wd, idesc, 1);
+          if (T32) {
+            ptx::mma_tf32_ss(d, ah + a_off, wd, idesc_wide, s != 0);
+            ptx::mma_tf32_ss(d + p.np, al + a_off, wd, idesc, 1);
+          } else {
+            ptx::mma_f16_ss(d, ah + a_off, wd, idesc_wide, s != 0);
+            ptx::mma_f16_ss(d + p.np, al + a_off, wd, idesc, 1);
+          }
         }
         ptx::tc_commit(&sh.a_empty[buf]);
         ptx::tc_commit(&sh.d_full[buf]);
@@ -346,7 +371,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
     const uint32_t lane_addr = tmem + (uint32_t((warp & 3) * 32) << 16);
     const int q = MODE == KDFT_CONTIG ? row % Q : row / L;
     const unsigned line = MODE == KDFT_CONTIG ? row / Q : row % L;
-    const uint64_t down11 = dup2(0x1p-11f);
+    const uint64_t down11 = dup2(T32 ? 1.0f : 0x1p-11f);
     // one factor where it is a normal number, else the two one after the other
     const float both = p.out_mul * out_mul2;
     const bool one_step = both > 1e-30f && both < 1e30f;
@@ -413,7 +438,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    if (lane == 0 && amax > 0.0f) atomicMax(p.amax_out, __float_as_uint(amax));
+    if (!T32 && lane == 0 && amax > 0.0f) atomicMax(p.amax_out, __float_as_uint(amax));
   } else {
     // -------------------------------------------------------------- load, R-point sums, phase, split
     ptx::setmaxnreg_inc<112>();
@@ -515,7 +540,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
           for (int s = 0; s < R; ++s) x[b][s] = {mul2(x[b][s].re, dup2(pre)), mul2(x[b][s].im, dup2(pre))};
       }
       {
-        const uint32_t col = grp * (B * 4);                        // bytes along the contraction (two halves per point)
+        const uint32_t col = grp * (B * (T32 ? 8 : 4));            // bytes along the contraction
         const uint32_t chunk = (col >> 4) & 7, low = col & 15;
         const uint32_t at0 = a_base + buf * 2 * piece_bytes + (col >> 7) * kFoldPanelBytes + low +
                              (MODE == KDFT_CONTIG ? line * Q * 128 : line * 128);
@@ -535,8 +560,8 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
             for (int q = h * Q; q < (h + 1) * Q; ++q) {
               // row (operand lane): line * R + q or q * L + line; the swizzle XORs the 16-byte chunk with row & 7
               const uint32_t sw = MODE == KDFT_CONTIG ? (line * Q + q) & 7 : line & 7;
-              const uint32_t at = at0 + h * 2 * piece_bytes + (q - h * Q) * (MODE == KDFT_CONTIG ? 128 : L * 128) +
-                                  ((chunk ^ sw) << 4);
+              const uint32_t row_at = at0 + h * 2 * piece_bytes + (q - h * Q) * (MODE == KDFT_CONTIG ? 128 : L * 128);
+              const uint32_t at = row_at + ((chunk ^ sw) << 4);
 #pragma unroll
               for (int b = 0; b < B / 2; ++b) {
                 uint64_t c, d, dn;
@@ -548,9 +573,18 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
                   lds_64(tn_at + (uint32_t(q) * p.mp / 2 + b) * 8, dn);
                   u = c2_mul(x[b][q], c, d, dn);
                 }
-                split_half2_scaled(u, hi[2 * b], hi[2 * b + 1], lo[2 * b], lo[2 * b + 1]);
+                if constexpr (T32) {           // two points fill a chunk of 16 bytes
+                  uint32_t th[4], tl[4];
+                  split_tf32(u, th, tl);
+                  const uint32_t to = row_at + (((chunk + b) ^ sw) << 4);
+                  sts_128(to, th[0], th[1], th[2], th[3]);
+                  sts_128(to + piece_bytes, tl[0], tl[1], tl[2], tl[3]);
+                } else {
+                  split_half2_scaled(u, hi[2 * b], hi[2 * b + 1], lo[2 * b], lo[2 * b + 1]);
+                }
               }
-              if constexpr (B == 4) {
+              if constexpr (T32) {
+              } else if constexpr (B == 4) {
                 sts_128(at, hi[0], hi[1], hi[2], hi[3]);
                 sts_128(at + piece_bytes, lo[0], lo[1], lo[2], lo[3]);
               } else {

@@ -1,4 +1,4 @@
-"""The folded form of uniform KDFT axes (csrc/fold_kernel.cuh): n = R*m with R = 4, 8 or 16 and m <= 64.
+"""The folded form of uniform axes (csrc/fold_kernel.cuh): n = R*m with R = 4, 8 or 16 and m <= 64 (TF32 pieces: 32).
 
 Bound: both operands carry 22 bits (2^-23 relative rounding each), sums and phases are fp32 (2^-24 per operation), the
 chains truncate at most 24 times: below 4e-7 per axis in the 2-norm; 1e-6 is asserted for up to three axes.
@@ -49,6 +49,49 @@ def test_folded_axes_against_the_oracle(lib, oracle, shape, sign):
     guard2 = torch.full((1 << 14,), 7.0, device="cuda")
     assert oracle.rel_l2(y.cpu().numpy(), oracle.dft3d(x.cpu().numpy(), sign=sign, scaled_inverse=sign > 0)) < BOUND
     assert bool((guard == 7.0).all()) and bool((guard2 == 7.0).all())
+
+
+# TF32 pieces: R and m as they fall there, groups and K = 8 steps with remainders, beside axes that are not folded (odd, and
+# more than 512 points), and the FFT formulation's 256 and 512 points with and without the blocked order and in place
+@pytest.mark.parametrize("mode,shape,axes", [("kdft", (100, 8, 4), None), ("kdft", (4, 128, 36), None), ("kdft", (252, 5, 12), None),
+                                             ("kdft", (20, 256, 16), None), ("kdft", (500, 4, 6), None), ("kdft", (4, 512, 8), None),
+                                             ("kdft", (3, 2, 496), None), ("kdft", (520, 12, 512), None), ("kdft", (64, 100, 32), None),
+                                             ("fft", (256, 512, 256), None), ("fft", (64, 512, 64), (1,)),
+                                             ("fft", (512, 64, 64), (0,)), ("fft", (3, 256, 512), (1, 2))])
+@pytest.mark.parametrize("sign", [-1, +1])
+def test_folded_axes_with_tf32_pieces(lib, oracle, mode, shape, axes, sign):
+    from paper_2002_03260_b200 import inputs
+    x = inputs.cube(shape, "normal", 305, device="cuda")
+    kw = dict(mode=lib.DFT3D_FFT if mode == "fft" else lib.DFT3D_KDFT, sign=sign, flags=lib.DFT3D_SPLIT_TF32, axes=axes)
+    y = _run(lib, x, **kw)
+    want = x.cpu().numpy().astype(np.complex128)
+    for a in axes or (0, 1, 2):
+        want = oracle.dft_axis(want, a, sign=sign, scale=1.0 / shape[a] if sign > 0 else 1.0)
+    folded = all(shape[a] % 4 == 0 and shape[a] <= 512 for a in axes or (0, 1, 2))
+    assert oracle.rel_l2(y.cpu().numpy(), want) < (BOUND if folded else 5e-6)   # 2e-6 per axis with the full matrix
+    if mode == "fft" and axes is None:
+        in_place = _run(lib, x, workspace_limit=1, **kw)
+        assert _rel(in_place, y) < BOUND
+
+
+# 512-point axes of FFT plans that leave the pieces open, in every schedule they appear in: beside axes that keep fp16 pieces
+# (whose blocked orders they share), in slices of the last axis, in place, alone, and after a KDFT axis; against the plan
+# that insists on fp16 pieces
+@pytest.mark.parametrize("shape,mode,axes,limit", [((512, 256, 64), "fft", None, 0), ((256, 512, 128), "fft", None, 0),
+                                                   ((512, 512, 256), "fft", None, 1 << 28), ((512, 256, 256), "fft", None, 1 << 26),
+                                                   ((1024, 512, 256), "fft", None, 1 << 28), ((512, 512, 512), "fft", None, 1),
+                                                   ((512, 2048, 64), "fft", None, 0), ((2048, 512, 64), "fft", None, 0),
+                                                   ((5, 512, 512), "fft", (1, 2), 0), ((12, 512, 256), "auto", None, 0)])
+def test_512_point_fft_axes(lib, shape, mode, axes, limit):
+    from paper_2002_03260_b200 import inputs
+    if mode == "fft" and axes is None and shape[2] % 256:
+        axes = (0, 1)
+    x = inputs.cube(shape, "normal", 306, device="cuda")
+    kw = dict(mode=lib.DFT3D_FFT if mode == "fft" else lib.DFT3D_AUTO, axes=axes, workspace_limit=limit)
+    y = _run(lib, x, **kw)
+    assert _rel(y, _run(lib, x, flags=lib.DFT3D_SPLIT_FP16, **kw)) < BOUND
+    if axes is None and mode == "fft":             # the transform itself, in 64 bits
+        assert _rel(y, torch.fft.fftn(x.to(torch.complex128))) < BOUND
 
 
 # the full matrix, which an axis with (uniform) nodes given keeps, in every form a plan takes
