@@ -138,7 +138,7 @@ __device__ __forceinline__ void fft_f16_axis_body(const CUtensorMap* map_data_p,
   const CUtensorMap& map_out = *map_out_p;
   const FftParams& p = pp.base;
   extern __shared__ uint8_t smem_raw_[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw_) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = ptx::align_1024(smem_raw_);
   constexpr int K = 2 * R;             // reals per contraction
   constexpr int NB = 2 * R;            // MMA N: the 2R output reals (k, re/im) of one stage
   constexpr int KS = K / 16;           // K = 16 steps per product

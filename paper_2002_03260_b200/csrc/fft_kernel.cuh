@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kFftThreads, 1)
 fft_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid_constant__ CUtensorMap map_w,
                 const __grid_constant__ CUtensorMap map_out, const FftParams p) {
   extern __shared__ uint8_t smem_raw_[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw_) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = ptx::align_1024(smem_raw_);
   constexpr int K = 2 * R;             // reals per contraction
   constexpr int NB = 2 * R;            // MMA N: the 2R output reals (k, re/im) of one stage
   constexpr int kWPiece = (K / 32) * NB * 128;   // bytes of one table piece in shared memory

@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
   constexpr int B = fold_group(R);  // consecutive i a thread takes at a time
   constexpr int kLog2R = R == 4 ? 2 : (R == 8 ? 3 : 4);
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = ptx::align_1024(smem_raw);
   uint8_t* smem_w = smem;
   uint8_t* smem_a = smem + p.w_bytes;                    // [buffer][hi, lo'][panel][128 rows][128 B]
   const uint32_t piece_bytes = uint32_t(p.panels) * kFoldPanelBytes;

@@ -111,7 +111,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kKdftThreads, 1)
 kdft_f16x2_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid_constant__ CUtensorMap map_w,
                  const KdftF16Params p) {
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = ptx::align_1024(smem_raw);
   uint8_t* smem_b = smem;
   uint8_t* smem_a = smem + size_t(kX2StagesB) * kX2BytesStageB;
   KdftX2Shared& sh = *reinterpret_cast<KdftX2Shared*>(smem_a + size_t(kX2StagesA) * kF16BytesStageA);

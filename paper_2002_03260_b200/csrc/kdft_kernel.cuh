@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(kKdftThreads, 1)
 kdft_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid_constant__ CUtensorMap map_w,
                  const KdftParams p) {
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* smem = ptx::align_1024(smem_raw);
   uint8_t* smem_b = smem;
   uint8_t* smem_a = smem + size_t(kStagesB) * kBytesStageB;
   KdftShared& sh = *reinterpret_cast<KdftShared*>(smem_a + size_t(kStagesA) * kBytesStageA);

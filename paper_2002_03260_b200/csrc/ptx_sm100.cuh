@@ -16,6 +16,10 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// the first 1024-byte boundary in dynamic shared memory; an offset, not a rounded pointer, so that the compiler still knows
+// the address space and emits shared-memory instead of generic loads and stores
+__device__ __forceinline__ uint8_t* align_1024(uint8_t* smem) { return smem + ((1024u - (smem_u32(smem) & 1023u)) & 1023u); }
+
 __device__ __forceinline__ bool elect_one() {
   uint32_t pred = 0;
   asm volatile(
