@@ -493,7 +493,11 @@ def main():
                         "bytes": "8 B read + 8 B written per point per axis pass (the reduction over the input comes on top)"}
             if split == dft.DFT3D_SPLIT_FP16:
                 paired = max(shape[a] for a in taxes) >= 2048 and os.environ.get("DFT3D_KDFT_PAIR", "1") != "0"
-                kernel = "kdft_f16x2_axis_kernel" if paired else "kdft_f16_axis_kernel"   # CTA pairs from 2048 points up
+                kernel = "kdft_f16x2_axis_kernel" if paired else "kdft_real_axis_kernel"   # CTA pairs from 2048 points up
+                if not paired:                      # a real matrix on real and imaginary parts: half the multiplications
+                    algo_flops *= 0.5
+                    issued *= 0.5
+                    ach *= 0.5
                 peak = peaks["bf16_tflops_sustained"]
                 src = "%s bf16 sustained (fp16 and bf16 share the tensor rate)" % peak_kind
                 axis_launches = nlaunch - 1
@@ -507,7 +511,7 @@ def main():
                     "traffic_note": "DRAM bytes per launch, ncu capture (%s) scaled by points (algorithmic: 16 B/point)"
                                     % dram_bytes_per_point(kernel)[1],
                     "peak_source": src,
-                    "flops": "issued tensor flops = 3 split products x 8*n_a flops per point per axis",
+                    "flops": "issued tensor flops = 3 split products x 8*n_a (real matrix: 4*n_a) flops per point per axis",
                     "useful_gemm_tflops": algo_flops / (ms * 1e-3) * 1e-12, "avg_launch_ms": ms / axis_launches}
 
         if mode == "kdft":

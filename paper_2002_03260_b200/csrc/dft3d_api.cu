@@ -19,6 +19,7 @@
 #include "generator.h"
 #include "kdft_kernel.cuh"
 #include "kdft_f16_kernel.cuh"
+#include "kdft_real_kernel.cuh"
 #include "fold_kernel.cuh"
 #include "fft_f16_kernel.cuh"
 #include "kdft_f16x2_kernel.cuh"
@@ -170,6 +171,10 @@ struct KdftAxis {
   bool pair = false;      // the paired-CTA kernel applies (fp16 pieces, 2n >= 256)
   int bn = 0;
   float out_mul = 1.0f;   // fp16 pieces: 2^-10, times 1/n for a scaled inverse
+  // fp16 pieces, axes of fewer than 2048 points: real table about the centre of the frequencies (kdft_real_kernel.cuh)
+  int form = 0;                  // 1 or 2; 0 = not in this form
+  float* d_phase = nullptr;
+  int phase_pitch = 0;
   // uniform grid, n = fold_r * m: the matrix in folded form (fold_kernel.cuh); 0 = not folded
   int fold_r = 0;
   bool fold_t32 = false;         // with TF32 pieces
@@ -282,10 +287,14 @@ int set_kernel_attributes(int device) {
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(dft3d::kKdftSmemBytes)));
   DFT3D_CUDA(cudaFuncSetAttribute(dft3d::kdft_axis_kernel<dft3d::KDFT_STRIDED>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(dft3d::kKdftSmemBytes)));
-  DFT3D_CUDA(cudaFuncSetAttribute(dft3d::kdft_f16_axis_kernel<dft3d::KDFT_CONTIG>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(dft3d::kKdftF16SmemBytes)));
-  DFT3D_CUDA(cudaFuncSetAttribute(dft3d::kdft_f16_axis_kernel<dft3d::KDFT_STRIDED>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(dft3d::kKdftF16SmemBytes)));
+  DFT3D_CUDA(cudaFuncSetAttribute(dft3d::kdft_real_axis_kernel<dft3d::KDFT_CONTIG, 1>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(dft3d::kKdftRealSmemBytes)));
+  DFT3D_CUDA(cudaFuncSetAttribute(dft3d::kdft_real_axis_kernel<dft3d::KDFT_CONTIG, 2>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(dft3d::kKdftRealSmemBytes)));
+  DFT3D_CUDA(cudaFuncSetAttribute(dft3d::kdft_real_axis_kernel<dft3d::KDFT_STRIDED, 1>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(dft3d::kKdftRealSmemBytes)));
+  DFT3D_CUDA(cudaFuncSetAttribute(dft3d::kdft_real_axis_kernel<dft3d::KDFT_STRIDED, 2>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, int(dft3d::kKdftRealSmemBytes)));
   DFT3D_CUDA(cudaFuncSetAttribute(dft3d::kdft_f16x2_axis_kernel<dft3d::KDFT_CONTIG>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(dft3d::kKdftX2SmemBytes)));
   DFT3D_CUDA(cudaFuncSetAttribute(dft3d::kdft_f16x2_axis_kernel<dft3d::KDFT_STRIDED>,
@@ -407,6 +416,81 @@ int build_fold_axis(dft3d_plan_s* p, KdftAxis& ax, int r, bool t32, double scale
   return DFT3D_OK;
 }
 
+// Tables of an axis in the real form (kdft_real_kernel.cuh): fp16 pieces of 2^s * R, n rows padded to 16 bytes, and the
+// phases.  `inverse` is NULL, or for a solve the n x n complex inverse of the forward matrix of the nodes: its real
+// factor about the centre follows from it, with the halves of the pair sums (form 2) or differences (form 1) included.
+int build_real_axis(dft3d_plan_s* p, KdftAxis& ax, const double* nodes, const double* inverse, double scale) {
+  const long long n = ax.n, ld = (n + 7) / 8 * 8;
+  const bool on_output = nodes && (p->flags & DFT3D_NODES_ON_OUTPUT);
+  ax.form = on_output == (inverse == nullptr) ? 2 : 1;
+  ax.bn = int(n < 256 ? (n + 15) / 16 * 16 : 256);
+  ax.phase_pitch = int((n + 63) / 64 * 64);
+  const size_t piece = size_t(n) * ld;
+  std::vector<double> T, ph;                              // T[row][column] as the kernel multiplies by it
+  std::vector<__half> H;
+  std::vector<float> phf;
+  try {
+    T.resize(size_t(n) * n);
+    ph.resize(size_t(2) * n);
+    H.assign(2 * piece, __float2half_rn(0.0f));
+    phf.assign(ax.form == 1 ? size_t(4) * ax.phase_pitch : size_t(2) * ((n + 255) / 256 * 256), 0.0f);
+  } catch (const std::bad_alloc&) {
+    return fail(DFT3D_ERR_ALLOC, "host allocation of a real axis table failed");
+  }
+  dft3d::gen::centre_phase(n, p->sign, nodes, ph.data());
+  double mx = 1.0;
+  if (!inverse) {
+    dft3d::gen::centred_matrix(n, nodes, T.data());
+    if (ax.form == 2)
+      for (long long i = 0; i < n; ++i)
+        for (long long j = 0; j < i; ++j) std::swap(T[i * n + j], T[j * n + i]);
+  } else {
+    mx = 0.0;
+    for (long long q = 0; q < n / 2; ++q)
+      for (long long j = 0; j < n; ++j) {                 // j: the index that carries the node
+        const long long r = n / 2 + q, l = n / 2 - 1 - q;
+        const double* vr = inverse + 2 * (ax.form == 2 ? j * n + r : r * n + j);
+        const double* vl = inverse + 2 * (ax.form == 2 ? j * n + l : l * n + j);
+        const double dr = ph[2 * j], di = -ph[2 * j + 1];                    // exp(-2*pi*i*c*t_j)
+        const double sr = vr[0] + vl[0], si = vr[1] + vl[1], tr = vr[0] - vl[0], ti = vr[1] - vl[1];
+        const double c = 0.5 * (sr * dr - si * di);                          // Re of (v_r + v_l) * d / 2
+        const double s = 0.5 * (tr * di + ti * dr);                          // Re of -i * (v_r - v_l) * d / 2
+        T[ax.form == 2 ? j * n + 2 * q : 2 * q * n + j] = c;
+        T[ax.form == 2 ? j * n + 2 * q + 1 : (2 * q + 1) * n + j] = s;
+        mx = std::fmax(mx, std::fmax(std::fabs(c), std::fabs(s)));
+      }
+  }
+  const int s2 = inverse ? 9 - std::ilogb(mx) : 10;       // largest table entry in [512, 1024]
+  const double tscale = std::ldexp(1.0, s2);
+  for (long long i = 0; i < n; ++i)
+    for (long long j = 0; j < n; ++j) {
+      const double v = tscale * T[i * n + j], hi = dft3d::gen::round_to_fp16(v);
+      H[i * ld + j] = __float2half_rn(float(hi));
+      H[piece + i * ld + j] = __float2half_rn(float(dft3d::gen::round_to_fp16(v - hi)));
+    }
+  for (long long j = 0; j < n; ++j) {
+    const float re = float(ph[2 * j]), im = float(ph[2 * j + 1]);
+    if (ax.form == 1) {                                   // z = re*a + im*b: (re, -im) for the real lane, (im, re) for the other
+      phf[2 * j] = re;
+      phf[2 * j + 1] = -im;
+      phf[2 * (ax.phase_pitch + j)] = im;
+      phf[2 * (ax.phase_pitch + j) + 1] = re;
+    } else {
+      phf[2 * j] = re;
+      phf[2 * j + 1] = im;
+    }
+  }
+  ax.out_mul = float((inverse ? 1.0 : scale) / tscale);
+  DFT3D_CUDA(cudaMalloc(&ax.d_w, H.size() * sizeof(__half)));
+  DFT3D_CUDA(cudaMemcpy(ax.d_w, H.data(), H.size() * sizeof(__half), cudaMemcpyHostToDevice));
+  DFT3D_CUDA(cudaMalloc(&ax.d_phase, phf.size() * sizeof(float)));
+  DFT3D_CUDA(cudaMemcpy(ax.d_phase, phf.data(), phf.size() * sizeof(float), cudaMemcpyHostToDevice));
+  const unsigned long long dims[3] = {(unsigned long long)n, (unsigned long long)n, 2ull};
+  const unsigned long long strides[2] = {(unsigned long long)(ld * 2), (unsigned long long)(piece * 2)};
+  const unsigned box[3] = {unsigned(dft3d::kF16BlockK), unsigned(ax.bn), 2u};
+  return encode_map(&ax.map_w, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, ax.d_w, 3, dims, strides, box, 128);
+}
+
 int build_kdft_axis(dft3d_plan_s* p, int a, const double* nodes) {
   KdftAxis& ax = p->kax[a];
   const long long n = p->n[a];
@@ -436,6 +520,11 @@ int build_kdft_axis(dft3d_plan_s* p, int a, const double* nodes) {
       return fail(DFT3D_ERR_UNSUPPORTED, "axis %d: the nodes make the system too ill-conditioned for fp32 data "
                   "(|V| |V^-1| = %.3g)", a, growth);
   }
+  // Pairs of CTAs (cta_group::2, kdft_f16x2_kernel.cuh) on the complex matrix from n = 2048 on, where a table no longer sits in
+  // L2 beside the data and the part runs at its 1 kW cap: every table tile is fetched once per pair.  Below, the real form.
+  const int pair_env = p->knobs.kdft_pair;
+  ax.pair = p->f16 && 2 * n >= 256 && (p->sm_count % 2 == 0) && (pair_env >= 0 ? pair_env != 0 : n >= 2048);
+  if (p->f16 && !ax.pair) return build_real_axis(p, ax, nodes, solve ? M.data() : nullptr, scale);
   if (p->f16) {
     // fp16 pieces of 2^s*W (s = 10 for entries of modulus one); the 1/n of a scaled inverse goes into the epilogue
     // multiplier instead of the table
@@ -472,22 +561,8 @@ int build_kdft_axis(dft3d_plan_s* p, int a, const double* nodes) {
     DFT3D_CUDA(cudaMemcpy(ax.d_w, H.data(), H.size() * sizeof(__half), cudaMemcpyHostToDevice));
     const unsigned long long hdims[3] = {(unsigned long long)(2 * n), (unsigned long long)(2 * n), 2ull};
     const unsigned long long hstrides[2] = {(unsigned long long)(2 * n * 2), (unsigned long long)(4 * n * n * 2)};
-    const unsigned hbox[3] = {unsigned(dft3d::kF16BlockK), unsigned(ax.bn), 2u};
-    {
-      // pairs of CTAs (cta_group::2) share a 256-column table tile, each loading 128 of its rows
-      const int env = p->knobs.kdft_pair;
-      // Same bits as the one-CTA kernel.  Its MMAs run at full rate but every chain end waits for a cross-CTA round
-      // trip, which cancels out at n = 1024 (77.6 vs 78.5 ms); at n = 2048, where the 64 MiB table no longer sits in
-      // L2 beside the data and the part runs at its 1 kW cap, fetching every table tile once per CTA pair wins
-      // (1365 -> 1235 ms, 1305 -> 1522 MHz).  Default: pairs from n = 2048 on.
-      ax.pair = ax.bn == 256 && (p->sm_count % 2 == 0) && (env >= 0 ? env != 0 : n >= 2048);
-      if (ax.pair) {
-        const unsigned pbox[3] = {unsigned(dft3d::kF16BlockK), 128u, 2u};
-        int rc = encode_map(&ax.map_w_pair, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, ax.d_w, 3, hdims, hstrides, pbox, 128);
-        if (rc != DFT3D_OK) return rc;
-      }
-    }
-    return encode_map(&ax.map_w, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, ax.d_w, 3, hdims, hstrides, hbox, 128);
+    const unsigned pbox[3] = {unsigned(dft3d::kF16BlockK), 128u, 2u};
+    return encode_map(&ax.map_w_pair, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, ax.d_w, 3, hdims, hstrides, pbox, 128);
   }
   if (!solve) dft3d::gen::axis_matrix(n, p->sign, scale, nodes, (p->flags & DFT3D_NODES_ON_OUTPUT) != 0, M.data());
   dft3d::gen::real_table_from_matrix(n, M.data(), W.data(), W.data() + size_t(4) * n * n);
@@ -517,8 +592,8 @@ int build_kdft_axis(dft3d_plan_s* p, int a, const double* nodes) {
 // Launches a kernel that may start while its predecessor in the stream drains (see ptx::griddep_wait): its set-up, the
 // launch latency and the predecessor's last CTAs overlap.  64^3 KDFT 27.7 -> 19.4 us, 64 x 128 x 192 with solved axes 65.6 ->
 // 53.3 us, 100 x 66 x 250 65.6 -> 60.9 us (the first two with the words of the scales cleared by the reduction instead
-// of a memset).  Cubes above 256 MiB gain nothing and lost up to 0.8 %: ordinary launches there.
-constexpr long long kOverlapPoints = 1ll << 25;
+// of a memset).  Cubes above 128 MiB gain nothing and lost up to 1 %: ordinary launches there.
+constexpr long long kOverlapPoints = 1ll << 24;
 template <class... Params, class... Args>
 cudaError_t launch_overlapped(const dft3d_plan_s* p, void (*kernel)(Params...), int grid, int threads, size_t smem,
                               cudaStream_t stream, Args&&... args) {
@@ -553,6 +628,69 @@ void fill_f16_params(Params& fp, const dft3d::KdftParams& kp, const KdftAxis& ax
   fp.n_group = p->knobs.kdft_ngroup >= 0 ? p->knobs.kdft_ngroup : ((kp.n_tiles >= 16 && ax.pair) ? 8 : 0);
 }
 
+// One pass in the real form; the lines of axis 2 are `batches` rows, those of axes 0 and 1 the columns of a
+// [batches][n][C] view.
+int launch_kdft_real(dft3d_plan_s* p, int a, const float* in, float* out, long long batches, long long C, cudaStream_t stream,
+                     int chain_pos) {
+  const KdftAxis& ax = p->kax[a];
+  const long long J = ax.n;
+  dft3d::KdftRealParams rp;
+  memset(&rp, 0, sizeof(rp));
+  rp.n = int(J);
+  rp.bn = ax.bn;
+  rp.n_tiles = int((J + ax.bn - 1) / ax.bn);
+  rp.chunk_kb = p->chunk_kb;
+  rp.phase = ax.d_phase;
+  rp.phase_pitch = ax.phase_pitch;
+  rp.sign = float(p->sign);
+  rp.out = out;
+  rp.status = p->d_status;
+  rp.out_mul = ax.out_mul;
+  rp.amax_in = p->d_amax + chain_pos;
+  rp.amax_out = p->d_amax + chain_pos + 1;
+  rp.wc = wait_control(p);
+  CUtensorMap map_data;
+  int rc;
+  if (a == 2) {
+    rp.rows = batches;
+    rp.m_tiles = (batches + dft3d::kRealLines - 1) / dft3d::kRealLines;
+    rp.lpb = dft3d::kRealLines;
+    rp.bpt = 1;
+    rp.c_tiles = 1;
+    rc = cached_map(p, &map_data, 0x120 + a, in, batches, 0, [&](CUtensorMap* m) {
+      const unsigned long long dims[2] = {(unsigned long long)(2 * J), (unsigned long long)batches};
+      const unsigned long long strides[1] = {(unsigned long long)(J * 8)};
+      const unsigned box[2] = {32u, unsigned(dft3d::kRealLines)};
+      return encode_f32(m, in, 2, dims, strides, box, 128);
+    });
+  } else {
+    rp.batches = batches;
+    rp.C = C;
+    rp.lpb = C <= 32 ? 32 : 64;    // columns beyond C are zero-filled and masked
+    rp.bpt = dft3d::kRealLines / rp.lpb;
+    rp.c_tiles = (C + rp.lpb - 1) / rp.lpb;
+    rp.m_tiles = rp.c_tiles * ((batches + rp.bpt - 1) / rp.bpt);
+    rc = cached_map(p, &map_data, 0x120 + a, in, batches, C, [&](CUtensorMap* m) {
+      const unsigned long long dims[3] = {(unsigned long long)(2 * C), (unsigned long long)J, (unsigned long long)batches};
+      const unsigned long long strides[2] = {(unsigned long long)(C * 8), (unsigned long long)(J * C * 8)};
+      const unsigned box[3] = {unsigned(2 * rp.lpb), ax.form == 1 ? 32u : 16u, unsigned(rp.bpt)};
+      return encode_f32(m, in, 3, dims, strides, box, 0, -1, p->knobs.promo_narrow);
+    });
+  }
+  if (rc != DFT3D_OK) return rc;
+  const long long total = rp.m_tiles * rp.n_tiles;
+  const int grid = int(total < p->sm_count ? total : p->sm_count);
+#define DFT3D_REAL_LAUNCH(MODE, FORM)                                                                              \
+  DFT3D_CUDA(launch_overlapped(p, dft3d::kdft_real_axis_kernel<MODE, FORM>, grid, dft3d::kKdftThreads,                \
+                               dft3d::kKdftRealSmemBytes, stream, map_data, ax.map_w, rp))
+  if (a == 2 && ax.form == 1) { DFT3D_REAL_LAUNCH(dft3d::KDFT_CONTIG, 1); }
+  else if (a == 2) { DFT3D_REAL_LAUNCH(dft3d::KDFT_CONTIG, 2); }
+  else if (ax.form == 1) { DFT3D_REAL_LAUNCH(dft3d::KDFT_STRIDED, 1); }
+  else { DFT3D_REAL_LAUNCH(dft3d::KDFT_STRIDED, 2); }
+#undef DFT3D_REAL_LAUNCH
+  return DFT3D_OK;
+}
+
 // chain_pos: position of this pass in the sequence of passes of one execute (fp16 pieces: which amax word to read)
 int launch_kdft_strided(dft3d_plan_s* p, int a, const float* in, float* out, long long batches, long long C,
                         cudaStream_t stream, int chain_pos) {
@@ -580,7 +718,7 @@ int launch_kdft_strided(dft3d_plan_s* p, int a, const float* in, float* out, lon
   int rc = cached_map(p, &map_data, 0x100 + a, in, batches, C, [&](CUtensorMap* m) {
     const unsigned long long dims[3] = {(unsigned long long)(2 * C), (unsigned long long)J, (unsigned long long)batches};
     const unsigned long long strides[2] = {(unsigned long long)(C * 8), (unsigned long long)(J * C * 8)};
-    // rows j per box: a whole stage for the paired-CTA kernel (32), half a stage for the one-CTA fp16 kernel, a TF32 stage (16)
+    // rows j per box: a stage of the paired-CTA kernel (32) or a TF32 stage (16)
     const unsigned box[3] = {unsigned(2 * kp.lpb), unsigned((f16 && ax.pair) ? dft3d::kF16BlockK / 2 : 16), unsigned(kp.bpt)};
     return encode_f32(m, in, 3, dims, strides, box, 0, -1, p->knobs.promo_narrow);
   });
@@ -594,11 +732,6 @@ int launch_kdft_strided(dft3d_plan_s* p, int a, const float* in, float* out, lon
     const int pgrid = 2 * int(pairs < p->sm_count / 2 ? pairs : p->sm_count / 2);
     dft3d::kdft_f16x2_axis_kernel<dft3d::KDFT_STRIDED>
         <<<pgrid, dft3d::kKdftThreads, dft3d::kKdftX2SmemBytes, stream>>>(map_data, ax.map_w_pair, fp);
-  } else if (f16) {
-    dft3d::KdftF16Params fp;
-    fill_f16_params(fp, kp, ax, p, chain_pos);
-    DFT3D_CUDA(launch_overlapped(p, dft3d::kdft_f16_axis_kernel<dft3d::KDFT_STRIDED>, grid, dft3d::kKdftThreads,
-                                 dft3d::kKdftF16SmemBytes, stream, map_data, ax.map_w, fp));
   } else {
     DFT3D_CUDA(launch_overlapped(p, dft3d::kdft_axis_kernel<dft3d::KDFT_STRIDED>, grid, dft3d::kKdftThreads,
                                  dft3d::kKdftSmemBytes, stream, map_data, ax.map_w, kp));
@@ -643,11 +776,6 @@ int launch_kdft_contig(dft3d_plan_s* p, int a, const float* in, float* out, long
     const int pgrid = 2 * int(pairs < p->sm_count / 2 ? pairs : p->sm_count / 2);
     dft3d::kdft_f16x2_axis_kernel<dft3d::KDFT_CONTIG>
         <<<pgrid, dft3d::kKdftThreads, dft3d::kKdftX2SmemBytes, stream>>>(map_data, ax.map_w_pair, fp);
-  } else if (p->f16) {
-    dft3d::KdftF16Params fp;
-    fill_f16_params(fp, kp, ax, p, chain_pos);
-    DFT3D_CUDA(launch_overlapped(p, dft3d::kdft_f16_axis_kernel<dft3d::KDFT_CONTIG>, grid, dft3d::kKdftThreads,
-                                 dft3d::kKdftF16SmemBytes, stream, map_data, ax.map_w, fp));
   } else {
     DFT3D_CUDA(launch_overlapped(p, dft3d::kdft_axis_kernel<dft3d::KDFT_CONTIG>, grid, dft3d::kKdftThreads,
                                  dft3d::kKdftSmemBytes, stream, map_data, ax.map_w, kp));
@@ -738,6 +866,11 @@ int kdft_axis_pass(dft3d_plan_s* p, int axis, const float* in, float* out, long 
   if (p->kax[axis].fold_r) {
     const long long lines = axis == 0 ? n1 * n2 : (axis == 1 ? planes * n2 : planes * n1);
     return launch_fold(p, axis, in, out, lines, axis == 0 ? n1 * n2 : (axis == 1 ? n2 : 1), stream, chain_pos, blocked);
+  }
+  if (p->kax[axis].form) {
+    if (axis == 0) return launch_kdft_real(p, 0, in, out, 1, n1 * n2, stream, chain_pos);
+    if (axis == 1) return launch_kdft_real(p, 1, in, out, planes, n2, stream, chain_pos);
+    return launch_kdft_real(p, 2, in, out, planes * n1, 0, stream, chain_pos);
   }
   if (axis == 0) return launch_kdft_strided(p, 0, in, out, 1, n1 * n2, stream, chain_pos);
   if (axis == 1) return launch_kdft_strided(p, 1, in, out, planes, n2, stream, chain_pos);
@@ -1824,6 +1957,7 @@ int dft3d_plan_destroy(dft3d_plan_t p) {
   if (!p) return DFT3D_OK;
   for (int a = 0; a < 3; ++a) {
     if (p->kax[a].d_w) cudaFree(p->kax[a].d_w);
+    if (p->kax[a].d_phase) cudaFree(p->kax[a].d_phase);
     if (p->kax[a].d_fold_w) cudaFree(p->kax[a].d_fold_w);
     if (p->kax[a].d_fold_tw) cudaFree(p->kax[a].d_fold_tw);
     if (p->fax[a].d_w) cudaFree(p->fax[a].d_w);

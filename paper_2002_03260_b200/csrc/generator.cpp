@@ -87,6 +87,26 @@ void axis_matrix(int64_t n, int sign, double scale, const double* nodes, bool no
 }
 
 namespace {
+// exp(2*pi*i * (twice/2) * t_j), t_j = nodes[j] or j/n
+void half_phasor(int64_t n, int64_t twice, const double* nodes, int64_t j, double* re, double* im) {
+  if (nodes) node_phasor(0.5 * static_cast<double>(twice), nodes[j], +1, re, im);
+  else root_of_unity(static_cast<int64_t>((static_cast<__int128>(twice) * j) % (2 * n)), 2 * n, +1, re, im);
+}
+}  // namespace
+
+void centred_matrix(int64_t n, const double* nodes, double* trig) {
+  for (int64_t p = 0; p < n / 2; ++p)
+    for (int64_t j = 0; j < n; ++j) half_phasor(n, 2 * p + 1, nodes, j, &trig[2 * p * n + j], &trig[(2 * p + 1) * n + j]);
+}
+
+void centre_phase(int64_t n, int sign, const double* nodes, double* phase) {
+  for (int64_t j = 0; j < n; ++j) {
+    half_phasor(n, n - 1, nodes, j, &phase[2 * j], &phase[2 * j + 1]);
+    if (sign < 0) phase[2 * j + 1] = -phase[2 * j + 1];
+  }
+}
+
+namespace {
 
 // all threads of a team meet here; sense-reversing spin barrier (the waits are microseconds long)
 struct SpinBarrier {

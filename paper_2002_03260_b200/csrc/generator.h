@@ -24,6 +24,12 @@ void axis_matrix(int64_t n, int sign, double scale, const double* nodes, bool no
 // max|matrix entry|, a cheap indication of how much accuracy the solve costs.
 bool invert_matrix(int64_t n, double* M, double* growth);
 
+// The axis matrix about its centre c = (n-1)/2 (n even): exp(+-2*pi*i*(c +- (p+1/2))*t_j) = exp(+-2*pi*i*c*t_j) *
+// (cos +- i*sin)(2*pi*(p+1/2)*t_j), with t_j = nodes[j], or j/n on a uniform grid.
+//   trig[2p][j], trig[2p+1][j] = cos, sin(2*pi*(p+1/2)*t_j)  (n x n reals);  phase[j] = exp(sign*2*pi*i*c*t_j) (n complex entries).
+void centred_matrix(int64_t n, const double* nodes, double* trig);
+void centre_phase(int64_t n, int sign, const double* nodes, double* phase);
+
 // T[k1][beta] = exp(sign*2*pi*i*k1*beta/(N1*N2))  (phase adjustment of Eq. 17), N1*N2 complex entries
 void twiddle(int64_t N1, int64_t N2, int sign, double* T);
 

@@ -1,0 +1,65 @@
+"""KDFT axes with nodes as products with a real matrix about the centre of the frequencies (csrc/kdft_real_kernel.cuh).
+
+Bound: the chain of the tensor core's accumulator is 48 products long, which truncates to about 1e-6 per axis (as with the
+complex matrix it replaces); 5e-6 is asserted for up to three axes, 2e-5 for a solve of jittered nodes (growth below 10).
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2002_03260_b200 as d
+    return d
+
+
+# a single quadruple, ragged stages (64 points), tiles (64 lines, 256 outputs) and batches, more than one table panel; the
+# uniform 260 points have no folded form and run here too
+@pytest.mark.parametrize("shape,axes", [((4, 8, 12), (0, 1, 2)), ((68, 60, 36), (0, 1, 2)), ((252, 20, 4), (0,)),
+                                        ((12, 260, 20), (1,)), ((5, 4, 516), (2,)), ((8, 516, 36), (1,)), ((260, 4, 100), (0,)),
+                                        ((2, 36, 256), (1, 2)), ((3, 128, 68), (1,))])
+@pytest.mark.parametrize("on_output", [False, True])
+@pytest.mark.parametrize("sign", [-1, +1])
+def test_nodes_on_single_axes(lib, oracle, shape, axes, on_output, sign):
+    from paper_2002_03260_b200 import inputs
+    x = inputs.cube(shape, "normal", 401, device="cuda")
+    full = inputs.sorted_nodes(shape, 402)
+    nodes = [full[a] * 3.0 - 1.0 if a in axes else None for a in range(3)]     # any finite value, used modulo 1
+    flags = lib.DFT3D_NODES_ON_OUTPUT if on_output else 0
+    guard = torch.full((1 << 14,), 7.0, device="cuda")
+    plan = lib.Plan(*shape, nodes=nodes, axes=axes, sign=sign, flags=flags)
+    y = plan(x)
+    torch.cuda.synchronize()
+    plan.status()
+    plan.destroy()
+    want = x.cpu().numpy().astype(np.complex128)
+    for a in axes:
+        want = oracle.dft_axis(want, a, sign=sign, scale=1.0 / shape[a] if sign > 0 else 1.0, nodes=nodes[a],
+                               nodes_on_output=on_output)
+    assert oracle.rel_l2(y.cpu().numpy(), want) < 5e-6
+    assert bool((guard == 7.0).all())
+
+
+@pytest.mark.parametrize("on_output", [False, True])
+@pytest.mark.parametrize("shape,axis", [((20, 12, 8), 0), ((4, 260, 12), 1), ((3, 5, 68), 2)])
+def test_solve_on_single_axes(lib, oracle, shape, axis, on_output):
+    from paper_2002_03260_b200 import inputs
+    x = inputs.cube(shape, "normal", 403, device="cuda")
+    n = shape[axis]
+    jitter = np.random.default_rng(404).uniform(-0.3, 0.3, n)
+    nodes = [None] * 3
+    nodes[axis] = (np.arange(n) + jitter) / n
+    flags = lib.DFT3D_INVERSE_SOLVE | (lib.DFT3D_NODES_ON_OUTPUT if on_output else 0)
+    plan = lib.Plan(*shape, nodes=nodes, axes=(axis,), sign=+1, flags=flags)
+    y = plan(x)
+    torch.cuda.synchronize()
+    plan.status()
+    plan.destroy()
+    want = oracle.solve_axis(x.cpu().numpy().astype(np.complex128), axis, nodes[axis], nodes_on_output=on_output)
+    assert oracle.rel_l2(y.cpu().numpy(), want) < 2e-5
