@@ -318,20 +318,22 @@ kdft_real_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid
     const float both = p.out_mul * out_mul2;
     const bool one_step = both > 1e-30f && both < 1e30f;
     const float mul = one_step ? both : p.out_mul, taum = tau * mul;
-    const uint32_t lane_addr = tmem + (uint32_t(q * 32) << 16) + half * 128;
-    const bool cols_active = half * 128 < p.bn;
+    const int width = ((p.bn + 1) / 2 + 31) / 32 * 32;       // columns of the first of the two halves, at most 128
+    const uint32_t lane_addr = tmem + (uint32_t(q * 32) << 16) + half * width;
     const int chunks_per_tile = (num_kb + p.chunk_kb - 1) / p.chunk_kb;
     uint32_t chunk_count = 0;
     for (long long t = blockIdx.x; t < total_tiles; t += gridDim.x) {
       const long long mt = t / p.n_tiles;
       const int nt = int(t % p.n_tiles);
+      const int c0 = nt * p.bn + half * width;   // first table column held by this thread
+      const int ncols = min(half ? p.bn - width : width, p.n - c0);   // how many of them (none or negative: none)
       float acc[128];
       for (int c = 0; c < chunks_per_tile; ++c, ++chunk_count) {
         DFT3D_WAIT_WARP(&sh.acc_full, chunk_count & 1, 0x401);
         ptx::tc_fence_after();
-        if (cols_active) {
 #pragma unroll
-          for (int g = 0; g < 4; ++g) {
+        for (int g = 0; g < 4; ++g) {
+          if (32 * g < ncols) {
             uint32_t v[32];
             ptx::tmem_ld_32x32(lane_addr + g * 32, v);
             ptx::tc_wait_ld();
@@ -349,9 +351,8 @@ kdft_real_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid
         if (lane == 0) ptx::mbar_arrive(&sh.acc_empty);
       }
       // ---- undo the scales, recombine the lanes of a line, note the largest magnitude for the next pass, store
-      const int c0 = nt * p.bn + half * 128;   // first table column held by this thread
       float amax = 0.0f;
-      if (cols_active && c0 < p.n) {
+      if (ncols > 0) {
         if (!one_step) {
 #pragma unroll
           for (int i = 0; i < 128; ++i) acc[i] *= out_mul2;
@@ -360,6 +361,7 @@ kdft_real_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid
           const float st = p.sign * taum;
 #pragma unroll
           for (int i = 0; i < 64; ++i) {
+            if (i / 16 * 32 >= ncols) break;
             const float other = __shfl_xor_sync(0xffffffffu, acc[2 * i + 1], 1), c = acc[2 * i] * mul;
             acc[2 * i] = fmaf(st, other, c);
             acc[2 * i + 1] = fmaf(-st, other, c);
@@ -368,6 +370,7 @@ kdft_real_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid
           const float4* ph = reinterpret_cast<const float4*>(p.phase) + c0 / 2;   // padded to whole tiles
 #pragma unroll
           for (int i = 0; i < 64; ++i) {
+            if (i / 16 * 32 >= ncols) break;
             const float4 f = __ldg(ph + i);
             const float o0 = __shfl_xor_sync(0xffffffffu, acc[2 * i], 1), o1 = __shfl_xor_sync(0xffffffffu, acc[2 * i + 1], 1);
             acc[2 * i] = fmaf(acc[2 * i] * mul, f.x, o0 * taum * f.y);
@@ -392,7 +395,7 @@ kdft_real_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid
             const long long hop = 2 * step * (FORM == 1 ? 1 : 2);
             float* up = p.out + 2 * (base + (FORM == 1 ? p.n / 2 + c0 / 2 : c0) * step) + comp;
             float* down = p.out + 2 * (base + (FORM == 1 ? p.n / 2 - 1 - c0 / 2 : c0 + 1) * step) + comp;
-            const int count = (p.n - c0) / 2;
+            const int count = ncols / 2;
             if (count >= 64) {
 #pragma unroll
               for (int i = 0; i < 64; ++i) {
@@ -419,6 +422,7 @@ kdft_real_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid
           float* dst = p.out + 2 * base;
 #pragma unroll
           for (int g = 0; g < 16; ++g) {
+            if (8 * g >= ncols) break;
 #pragma unroll
             for (int side = 0; side < 2; ++side) {
               // four outputs in ascending order, own part of each: this lane keeps w[2*comp], w[2*comp+1]
@@ -430,12 +434,12 @@ kdft_real_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid
 #pragma unroll
                 for (int i = 0; i < 4; ++i) w[i] = side == 0 ? acc[2 * (4 * g + i)] : acc[2 * (4 * g + 3 - i) + 1];
                 e = side == 0 ? p.n / 2 + p0 : p.n / 2 - 4 - p0;
-                ok = side == 0 ? p0 + 2 * comp < p.n / 2 : p0 + 2 - 2 * comp < p.n / 2;
+                ok = side == 0 ? p0 + 2 * comp < (c0 + ncols) / 2 : p0 + 2 - 2 * comp < (c0 + ncols) / 2;
               } else {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) w[i] = acc[8 * g + 4 * side + i];
                 e = c0 + 8 * g + 4 * side;
-                ok = e + 2 * comp < p.n;
+                ok = e + 2 * comp < c0 + ncols;
               }
               const float r0 = __shfl_xor_sync(0xffffffffu, comp ? w[0] : w[2], 1);
               const float r1 = __shfl_xor_sync(0xffffffffu, comp ? w[1] : w[3], 1);
