@@ -500,7 +500,11 @@ int build_kdft_axis(dft3d_plan_s* p, int a, const double* nodes) {
   const double scale = scaled ? 1.0 / double(n) : 1.0;
   // uniform grid: the folded form where the length has one (line numbers are 32-bit there)
   const int fold = fold_radix(n, p->f16);
-  if (!nodes && fold && points(p) / n < (1ll << 31)) return build_fold_axis(p, ax, fold, !p->f16, scale);
+  // The sizes that dft3d_kdft_execute_static takes too keep its kernel with TF32 pieces: a plan and a static call on the
+  // same tables agree to the bit.
+  const bool as_static = !p->f16 && p->axes == 7u && p->n[0] % 64 == 0 && p->n[1] % 64 == 0 && p->n[2] % 64 == 0 &&
+                         points(p) <= (1ll << 21);
+  if (!nodes && fold && !as_static && points(p) / n < (1ll << 31)) return build_fold_axis(p, ax, fold, !p->f16, scale);
   std::vector<double> M;
   std::vector<float> W;
   try {
