@@ -272,6 +272,10 @@ dft3d::WaitControl wait_control(const dft3d_plan_s* p) {
 int fold_radix(long long n, bool f16) {
   for (int r = 4; r <= 16; r *= 2)
     if (n % r == 0 && n / r <= (f16 ? 64 : 32)) return r;
+  // lengths that are no multiple of four run with TF32 pieces
+  const int other[6] = {1, 2, 3, 5, 6, 10};
+  for (int r : other)
+    if (!f16 && n % 4 != 0 && n % r == 0 && n / r <= 32) return r;
   return 0;
 }
 constexpr size_t kFoldSmemMax = dft3d::fold_smem_bytes(64 * 1024, 2, 1024);
@@ -345,6 +349,12 @@ int set_kernel_attributes(int device) {
   DFT3D_FOLD_ATTR(4, true);
   DFT3D_FOLD_ATTR(8, true);
   DFT3D_FOLD_ATTR(16, true);
+  DFT3D_FOLD_ATTR(1, true);
+  DFT3D_FOLD_ATTR(2, true);
+  DFT3D_FOLD_ATTR(3, true);
+  DFT3D_FOLD_ATTR(5, true);
+  DFT3D_FOLD_ATTR(6, true);
+  DFT3D_FOLD_ATTR(10, true);
 #undef DFT3D_FOLD_ATTR
   DFT3D_CUDA(cudaFuncSetAttribute(dft3d::fft_f16_fused_kernel<32, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   int(dft3d::fft16_smem_bytes(32, 1))));
@@ -838,20 +848,33 @@ int launch_fold(dft3d_plan_s* p, int a, const float* in, float* out, long long l
   const int grid = int(fp.units < unsigned(p->sm_count) ? fp.units : unsigned(p->sm_count));
   const size_t smem = dft3d::fold_smem_bytes(fp.w_bytes, fp.panels, r * fp.mp);
   const float sign = float(p->sign);
-#define DFT3D_FOLD_LAUNCH(MODE, R)                                                                                       \
-  DFT3D_CUDA(ax.fold_t32 ? launch_overlapped(p, dft3d::fold_axis_kernel<MODE, R, true>, grid, dft3d::kFoldThreads, smem,   \
-                                             stream, fp, sign)                                                            \
-                         : launch_overlapped(p, dft3d::fold_axis_kernel<MODE, R, false>, grid, dft3d::kFoldThreads, smem,  \
-                                             stream, fp, sign))
-  if (a == 2) {
-    if (r == 4) { DFT3D_FOLD_LAUNCH(dft3d::KDFT_CONTIG, 4); }
-    else if (r == 8) { DFT3D_FOLD_LAUNCH(dft3d::KDFT_CONTIG, 8); }
-    else { DFT3D_FOLD_LAUNCH(dft3d::KDFT_CONTIG, 16); }
+#define DFT3D_FOLD_LAUNCH(MODE, R, T32)                                                                               \
+  DFT3D_CUDA(launch_overlapped(p, dft3d::fold_axis_kernel<MODE, R, T32>, grid, dft3d::kFoldThreads, smem, stream, fp, sign))
+#define DFT3D_FOLD_CASE(R, T32)                                                      \
+  case R:                                                                            \
+    if (a == 2) { DFT3D_FOLD_LAUNCH(dft3d::KDFT_CONTIG, R, T32); }                   \
+    else { DFT3D_FOLD_LAUNCH(dft3d::KDFT_STRIDED, R, T32); }                         \
+    break;
+  if (ax.fold_t32) {
+    switch (r) {
+      DFT3D_FOLD_CASE(1, true)
+      DFT3D_FOLD_CASE(2, true)
+      DFT3D_FOLD_CASE(3, true)
+      DFT3D_FOLD_CASE(4, true)
+      DFT3D_FOLD_CASE(5, true)
+      DFT3D_FOLD_CASE(6, true)
+      DFT3D_FOLD_CASE(8, true)
+      DFT3D_FOLD_CASE(10, true)
+      DFT3D_FOLD_CASE(16, true)
+    }
   } else {
-    if (r == 4) { DFT3D_FOLD_LAUNCH(dft3d::KDFT_STRIDED, 4); }
-    else if (r == 8) { DFT3D_FOLD_LAUNCH(dft3d::KDFT_STRIDED, 8); }
-    else { DFT3D_FOLD_LAUNCH(dft3d::KDFT_STRIDED, 16); }
+    switch (r) {
+      DFT3D_FOLD_CASE(4, false)
+      DFT3D_FOLD_CASE(8, false)
+      DFT3D_FOLD_CASE(16, false)
+    }
   }
+#undef DFT3D_FOLD_CASE
 #undef DFT3D_FOLD_LAUNCH
   DFT3D_CUDA(cudaGetLastError());
   return DFT3D_OK;

@@ -73,13 +73,18 @@ struct FoldShared {
 constexpr int kFoldThreads = 640;
 constexpr int kFoldSplitWarps = 12;
 // consecutive i that a thread takes at a time
-__host__ __device__ constexpr int fold_group(int R) { return R == 16 ? 2 : 4; }
+__host__ __device__ constexpr int fold_group(int R) { return R >= 10 ? 2 : 4; }
 // A unit is the lines whose R-point sums are formed together, 32 warps' worth at most: one tile of 128 lanes (128/R lines
 // x R classes), or, on the strided axes with R = 16, two tiles of 16 lines x 8 classes, so that every row of the data is
 // read and written in pieces of at least a 128-byte line.  (With one tile of 8 lines the halves of the lines were fetched
 // from DRAM twice: 1.8 instead of 1.07 GB at 128 x 1024 x 1024, 652 us.)
-__host__ __device__ constexpr int fold_tiles(bool strided, int R) { return strided && R == 16 ? 2 : 1; }
-__host__ __device__ constexpr int fold_lines(bool strided, int R) { return 128 / R * fold_tiles(strided, R); }
+__host__ __device__ constexpr int fold_tiles(bool strided, int R) { return strided && R >= 10 ? 2 : 1; }
+// lines per unit: the largest power of two that 128 lanes hold (R = 3, 5, 6 and 10 leave some lanes idle)
+__host__ __device__ constexpr int fold_lines(bool strided, int R) {
+  int l = 1;
+  while (2 * l * (R / fold_tiles(strided, R)) <= 128) l *= 2;
+  return l;
+}
 constexpr int kFoldPanelBytes = 128 * 128;      // 128 lanes x 128 bytes
 __host__ __device__ constexpr size_t fold_smem_bytes(unsigned w_bytes, int panels, int tw_entries) {
   return size_t(w_bytes) + size_t(4) * panels * kFoldPanelBytes + size_t(tw_entries) * 12 + sizeof(FoldShared) + 1024;
@@ -113,6 +118,28 @@ __device__ __forceinline__ void dft4(C2& x0, C2& x1, C2& x2, C2& x3, uint64_t sp
   x1 = c2_add_i(b, d, sp, sn);
   x3 = c2_add_i(b, d, sn, sp);
 }
+__device__ __forceinline__ void dft3(C2& x0, C2& x1, C2& x2, uint64_t sp, uint64_t sn) {
+  const uint64_t half = dup2(-0.5f), h = dup2(0.86602540378443864676f);
+  const C2 t = c2_add(x1, x2), d = c2_sub(x1, x2), b = {mul2(d.re, h), mul2(d.im, h)};
+  const C2 a = {fma2(t.re, half, x0.re), fma2(t.im, half, x0.im)};
+  x0 = c2_add(x0, t);
+  x1 = c2_add_i(a, b, sp, sn);
+  x2 = c2_add_i(a, b, sn, sp);
+}
+__device__ __forceinline__ void dft5(C2& x0, C2& x1, C2& x2, C2& x3, C2& x4, uint64_t sp, uint64_t sn) {
+  const uint64_t c1 = dup2(0.30901699437494742410f), c2 = dup2(-0.80901699437494742410f);
+  const uint64_t s1 = dup2(0.95105651629515357212f), s2 = dup2(0.58778525229247312917f), s1n = dup2(-0.95105651629515357212f);
+  const C2 t1 = c2_add(x1, x4), t2 = c2_add(x2, x3), t3 = c2_sub(x1, x4), t4 = c2_sub(x2, x3);
+  const C2 a1 = {fma2(t2.re, c2, fma2(t1.re, c1, x0.re)), fma2(t2.im, c2, fma2(t1.im, c1, x0.im))};
+  const C2 a2 = {fma2(t2.re, c1, fma2(t1.re, c2, x0.re)), fma2(t2.im, c1, fma2(t1.im, c2, x0.im))};
+  const C2 b1 = {fma2(t4.re, s2, mul2(t3.re, s1)), fma2(t4.im, s2, mul2(t3.im, s1))};
+  const C2 b2 = {fma2(t4.re, s1n, mul2(t3.re, s2)), fma2(t4.im, s1n, mul2(t3.im, s2))};
+  x0 = c2_add(x0, c2_add(t1, t2));
+  x1 = c2_add_i(a1, b1, sp, sn);
+  x4 = c2_add_i(a1, b1, sn, sp);
+  x2 = c2_add_i(a2, b2, sp, sn);
+  x3 = c2_add_i(a2, b2, sn, sp);
+}
 __device__ __forceinline__ void c2_swap(C2& a, C2& b) { const C2 t = a; a = b; b = t; }
 
 // x[s] -> sum_s exp(sign*2*pi*i*s*q/R) x[s], natural order
@@ -120,7 +147,38 @@ template <int R>
 __device__ __forceinline__ void dft_r(C2 (&x)[R], float s) {
   constexpr float kC1 = 0.92387953251128675613f, kS1 = 0.38268343236508977173f, kH = 0.70710678118654752440f;
   const uint64_t sp = dup2(s), sn = dup2(-s);
-  if constexpr (R == 4) {
+  if constexpr (R == 2) {
+    const C2 a = x[0];
+    x[0] = c2_add(a, x[1]);
+    x[1] = c2_sub(a, x[1]);
+  } else if constexpr (R == 3) {
+    dft3(x[0], x[1], x[2], sp, sn);
+  } else if constexpr (R == 5) {
+    dft5(x[0], x[1], x[2], x[3], x[4], sp, sn);
+  } else if constexpr (R == 6 || R == 10) {     // even and odd points, then the odd half turned by exp(s*2*pi*i*q/R)
+    constexpr int K = R / 2;
+    constexpr float kCos[5] = {1.0f, R == 6 ? 0.5f : 0.80901699437494742410f, R == 6 ? -0.5f : 0.30901699437494742410f,
+                               -0.30901699437494742410f, -0.80901699437494742410f};
+    constexpr float kSin[5] = {0.0f, R == 6 ? 0.86602540378443864676f : 0.58778525229247312917f,
+                               R == 6 ? 0.86602540378443864676f : 0.95105651629515357212f, 0.95105651629515357212f,
+                               0.58778525229247312917f};
+    C2 e[K], o[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) { e[q] = x[2 * q]; o[q] = x[2 * q + 1]; }
+    if constexpr (K == 3) {
+      dft3(e[0], e[1], e[2], sp, sn);
+      dft3(o[0], o[1], o[2], sp, sn);
+    } else {
+      dft5(e[0], e[1], e[2], e[3], e[K - 1], sp, sn);
+      dft5(o[0], o[1], o[2], o[3], o[K - 1], sp, sn);
+    }
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+      const C2 t = q == 0 ? o[0] : c2_mul(o[q], dup2(kCos[q]), dup2(s * kSin[q]), dup2(-s * kSin[q]));
+      x[q] = c2_add(e[q], t);
+      x[q + K] = c2_sub(e[q], t);
+    }
+  } else if constexpr (R == 4) {
     dft4(x[0], x[1], x[2], x[3], sp, sn);
   } else if constexpr (R == 8) {
     dft4(x[0], x[2], x[4], x[6], sp, sn);
@@ -136,7 +194,7 @@ __device__ __forceinline__ void dft_r(C2 (&x)[R], float s) {
     x[6] = c2_add_i(e2, o2, sn, sp);
     x[3] = c2_add(e3, o3);
     x[7] = c2_sub(e3, o3);
-  } else {
+  } else if constexpr (R == 16) {
 #pragma unroll
     for (int a = 0; a < 4; ++a) dft4(x[a], x[a + 4], x[a + 8], x[a + 12], sp, sn);
     // x[a + 4*q0] *= w^(a*q0), w = exp(s*2*pi*i/16)
@@ -254,13 +312,13 @@ template <int MODE, int R, bool T32>
 __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldParams p, const float sign) {
   constexpr int H = fold_tiles(MODE == KDFT_STRIDED, R);   // tiles per unit
   constexpr int Q = R / H;          // residue classes per tile
-  constexpr int L = 128 / Q;        // lines per unit (and per tile)
+  constexpr int L = fold_lines(MODE == KDFT_STRIDED, R);   // lines per unit (and per tile)
   // How many units ahead the L2 prefetch runs, 64 or 128 KB per unit (512 x 1024 x 1024, microseconds per pass without the
   // reduction: strided R = 16 2147 / 1820 / 2040 / 2170 for no prefetch, 1, 2 and 3 units; contiguous R = 8 2270 / 1870 / 1720 /
   // 1860).
   constexpr unsigned kAhead = H == 2 ? 1 : 2;
   constexpr int B = fold_group(R);  // consecutive i a thread takes at a time
-  constexpr int kLog2R = R == 4 ? 2 : (R == 8 ? 3 : 4);
+  constexpr int kLog2R = R <= 4 ? 2 : (R <= 8 ? 3 : 4);    // at least log2(R)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = ptx::align_1024(smem_raw);
   uint8_t* smem_w = smem;
@@ -380,7 +438,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
     for (unsigned k = 0; k < my_tiles; ++k) {
       const uint32_t buf = k & 1, ph = (k >> 1) & 1;
       const unsigned l = (blockIdx.x + (k / H) * gridDim.x) * L + line;
-      const bool live = l < p.lines;
+      const bool live = l < p.lines && (MODE == KDFT_CONTIG ? line < unsigned(L) : q < Q);   // not an idle lane
       float2* dst;
       size_t step;
       if (MODE == KDFT_CONTIG) {
@@ -460,8 +518,9 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
         grp = id - line * p.groups;
       } else {
         // sixteen lines: eight of them and two groups per half warp, so that its 8-byte operand stores meet every bank once
-        line = L == 16 ? (lane & 7) | ((lane >> 4) << 3) : lane;
-        grp = L == 16 ? j * 2 + ((lane >> 3) & 1) : j;
+        constexpr unsigned kWarps = L > 32 ? L / 32 : 1;           // warps side by side
+        line = L == 16 ? (lane & 7) | ((lane >> 4) << 3) : (j % kWarps) * 32 + lane;
+        grp = L == 16 ? j * 2 + ((lane >> 3) & 1) : j / kWarps;
       }
       const bool mine = line < unsigned(L) && grp < p.groups;
       C2 x[B / 2][R];

@@ -56,6 +56,11 @@ def test_folded_axes_against_the_oracle(lib, oracle, shape, sign):
 @pytest.mark.parametrize("mode,shape,axes", [("kdft", (100, 8, 4), None), ("kdft", (4, 128, 36), None), ("kdft", (252, 5, 12), None),
                                              ("kdft", (20, 256, 16), None), ("kdft", (500, 4, 6), None), ("kdft", (4, 512, 8), None),
                                              ("kdft", (3, 2, 496), None), ("kdft", (520, 12, 512), None), ("kdft", (64, 100, 32), None),
+                                             # not multiples of four: R = 1, 2, 3, 5, 6 and 10, m up to 32, odd and even, alone or together
+                                             ("kdft", (31, 1, 2), None), ("kdft", (29, 25, 30), None), ("kdft", (62, 58, 54), None),
+                                             ("kdft", (93, 87, 6), None), ("kdft", (155, 5, 10), None), ("kdft", (66, 186, 6), None),
+                                             ("kdft", (250, 310, 4), None), ("kdft", (7, 3, 310), None), ("kdft", (9, 66, 250), None),
+                                             ("kdft", (3, 70, 190), (1, 2)), ("kdft", (5, 14, 186), (2,)), ("kdft", (66, 33, 18), (0,)),
                                              ("fft", (256, 512, 256), None), ("fft", (64, 512, 64), (1,)),
                                              ("fft", (512, 64, 64), (0,)), ("fft", (3, 256, 512), (1, 2))])
 @pytest.mark.parametrize("sign", [-1, +1])
@@ -67,7 +72,8 @@ def test_folded_axes_with_tf32_pieces(lib, oracle, mode, shape, axes, sign):
     want = x.cpu().numpy().astype(np.complex128)
     for a in axes or (0, 1, 2):
         want = oracle.dft_axis(want, a, sign=sign, scale=1.0 / shape[a] if sign > 0 else 1.0)
-    folded = all(shape[a] % 4 == 0 and shape[a] <= 512 for a in axes or (0, 1, 2))
+    radices = lambda n: (4, 8, 16) if n % 4 == 0 else (1, 2, 3, 5, 6, 10)
+    folded = all(any(shape[a] % r == 0 and shape[a] // r <= 32 for r in radices(shape[a])) for a in axes or (0, 1, 2))
     assert oracle.rel_l2(y.cpu().numpy(), want) < (BOUND if folded else 5e-6)   # 2e-6 per axis with the full matrix
     if mode == "fft" and axes is None:
         in_place = _run(lib, x, workspace_limit=1, **kw)
