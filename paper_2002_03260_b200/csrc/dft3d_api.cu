@@ -1161,7 +1161,9 @@ int fft_axis_pass(dft3d_plan_s* p, int axis, const float* in, float* out, cudaSt
     {
       // prefetching helps while rows are close (axis 1); with rows MiBs apart (axis 0) the pass is bound by the
       // rate of address translations and every extra request costs more than it hides (measured: 10.0 -> 12.2 ms)
-      fp.l2_prefetch = kn.fft_l2_prefetch >= 0 ? kn.fft_l2_prefetch : (C * 8 < (1ll << 20) ? 1 : 0);
+      // The fp16 kernel with R = 32 keeps up without (axis 1 of 100 x 1024 x 1024: 370 us without, 377 us with; 60 x 2048 x 1024
+      // 536 / 541; 8192 x 8192 914 / 933).
+      fp.l2_prefetch = kn.fft_l2_prefetch >= 0 ? kn.fft_l2_prefetch : (C * 8 < (1ll << 20) && !(p->f16 && R == 32) ? 1 : 0);
       if (n2_sub) fp.l2_prefetch = 0;
     }
     fp.mtiles_per_stage = cols / Lg;
