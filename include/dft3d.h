@@ -53,7 +53,8 @@ enum {
   /* Operand split of the tensor-core products (Section II-A: float32 accuracy from several reduced-precision
      pieces whose products are accumulated).  Both use 3
      products of 11-bit pieces with fp32 accumulation and meet the same error bound.  Default: fp16 pieces (KDFT:
-     when every transformed n_a % 4 == 0, TF32 pieces otherwise). */
+     when every transformed n_a % 4 == 0, TF32 pieces otherwise); FFT axes of 512 points take TF32 pieces unless fp16
+     ones are insisted on. */
   DFT3D_SPLIT_FP16 = 4u,        /* insist on fp16 pieces (operands scaled by exact powers of two: KDFT from the largest
                                    input magnitude, FFT per line; half the tensor-core instructions of TF32);
                                    DFT3D_ERR_UNSUPPORTED for KDFT when a transformed n_a is not a multiple of 4 */
@@ -107,6 +108,10 @@ typedef struct dft3d_options_s {
  *            Any finite value is accepted and used modulo 1.  Copied during the call.
  *            With nodes and sign=+1 the result is the conjugate-kernel product (see DFT3D_INVERSE_SOLVE), not an
  *            inverse of the nonuniform transform.  FFT mode takes no nodes.
+ *
+ * KDFT axes apply their matrix in the form that costs least: on a uniform grid with n_a = R*m (R = 4, 8 or 16 and m <= 64;
+ * TF32 pieces: also R = 1, 2, 3, 5, 6 or 10, m <= 32) the R residue classes of the output share one m x m matrix; with nodes
+ * and fp16 pieces below 2048 points a real matrix about the centre of the frequencies; otherwise the full matrix.
  *
  * The DFT / Vandermonde matrices and twiddles are evaluated in float64 with exactly
  * reduced phases and rounded once to the stored float32 pieces.  The plan owns its
@@ -183,7 +188,8 @@ size_t dft3d_plan_workspace_bytes(dft3d_plan_t plan);
  * 2 * slices + 1 when the workspace holds only a half, a quarter or an eighth of a cube. */
 int dft3d_plan_launches(dft3d_plan_t plan);
 
-/* DFT3D_SPLIT_FP16 or DFT3D_SPLIT_TF32: the operand split the plan uses; 0 for NULL. */
+/* DFT3D_SPLIT_FP16 or DFT3D_SPLIT_TF32: the operand split the plan uses (FFT axes of 512 points: see the flags); 0 for
+ * NULL. */
 int dft3d_plan_split(dft3d_plan_t plan);
 
 /* The factor pair {N1, N2} of Eq. 17 that the plan uses on `axis` (N1 * N2 = n_axis): DFT3D_OK and the pair for an axis

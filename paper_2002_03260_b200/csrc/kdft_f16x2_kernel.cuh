@@ -1,4 +1,4 @@
-// The KDFT axis kernel with fp16 pieces (kdft_f16_kernel.cuh) on PAIRS of CTAs: tcgen05.mma cta_group::2.
+// The KDFT axis kernel on the complex matrix with fp16 pieces (kdft_f16_kernel.cuh), on PAIRS of CTAs: tcgen05.mma cta_group::2.
 //
 // Two CTAs of a cluster (the two SMs of a TPC) work on one 256-lane x 256-column tile: each CTA owns 128 lanes (its own
 // raw data stages, split warps, tensor-memory A stages, accumulator and epilogue) and loads only HALF of every table
