@@ -390,6 +390,10 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
   const unsigned my_units = blockIdx.x < p.units ? (p.units - 1 - blockIdx.x) / gridDim.x + 1 : 0;
   const unsigned my_tiles = my_units * H;
 
+  // TF32 steps contract 8 instead of 16: twice as many additions that truncate.  Even and odd steps take accumulators of
+  // their own (np <= 64 there), which the epilogue adds in round-to-nearest fp32.
+  const bool twin = T32 && p.ks >= 2;
+
   if (warp < 4) {
     ptx::setmaxnreg_dec<40>();
     if (warp == 0 && lane == 0) {
@@ -411,8 +415,9 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
           const uint32_t a_off = uint32_t(s >> 2) * (kFoldPanelBytes >> 4) + (s & 3) * 2;
           const uint64_t wd = w0 + uint32_t(s >> 2) * w_panel + (s & 3) * 2;
           if (T32) {
-            ptx::mma_tf32_ss(d, ah + a_off, wd, idesc_wide, s != 0);
-            ptx::mma_tf32_ss(d + p.np, al + a_off, wd, idesc, 1);
+            const uint32_t dt = d + (twin && (s & 1) ? 128 : 0);
+            ptx::mma_tf32_ss(dt, ah + a_off, wd, idesc_wide, s > (twin ? 1 : 0));
+            ptx::mma_tf32_ss(dt + p.np, al + a_off, wd, idesc, 1);
           } else {
             ptx::mma_f16_ss(d, ah + a_off, wd, idesc_wide, s != 0);
             ptx::mma_f16_ss(d + p.np, al + a_off, wd, idesc, 1);
@@ -456,6 +461,17 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
         ptx::tmem_ld_32x32(lane_addr + buf * 256 + c0, hh);
         ptx::tmem_ld_32x32(lane_addr + buf * 256 + p.np + c0, xx);
         ptx::tc_wait_ld();
+        if (twin) {
+          uint32_t more[32];
+          ptx::tmem_ld_32x32(lane_addr + buf * 256 + 128 + c0, more);
+          ptx::tc_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 32; ++i) hh[i] = __float_as_uint(__uint_as_float(hh[i]) + __uint_as_float(more[i]));
+          ptx::tmem_ld_32x32(lane_addr + buf * 256 + 128 + p.np + c0, more);
+          ptx::tc_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 32; ++i) xx[i] = __float_as_uint(__uint_as_float(xx[i]) + __uint_as_float(more[i]));
+        }
         if (c0 + 32 >= 2 * p.m) {     // the accumulator has been read: the next tile may overwrite it
           ptx::tc_fence_before();
           __syncwarp();
