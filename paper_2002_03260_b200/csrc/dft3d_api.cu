@@ -956,9 +956,9 @@ int build_fft_axis(dft3d_plan_s* p, int a, const int split[2]) {
                                                                            // (fft_axis_pass may pick 8 for R = 32, RX = 1)
   // One product in folded form, with TF32 pieces, instead of two: always where the plan has TF32 pieces, and on 512-point axes
   // of plans that leave the pieces open (512^3, microseconds per pass, this against fp16 pieces: axis 0 491 / 577,
-  // axis 1 415 / 565, axis 2 394 / 428; no scaling and no larger error).  256 points: 58 to 63 against 59 to 69 at 256^3, which
-  // is too little to give up the arithmetic that the launch over axes 1 and 2 shares.
-  if (fold_radix(n, false) && (!p->f16 || (n == 512 && !(p->flags & DFT3D_SPLIT_FP16)))) {
+  // axis 1 415 / 565, axis 2 394 / 428; no scaling and no larger error).  256 points (256^3: 63 / 69, 59 / 68, 63 / 59): on axis 0
+  // only, since axes 1 and 2 keep the arithmetic that the launch over both of them shares.
+  if (fold_radix(n, false) && (!p->f16 || ((n == 512 || (n == 256 && a == 0)) && !(p->flags & DFT3D_SPLIT_FP16)))) {
     p->kax[a].n = n;
     return build_fold_axis(p, p->kax[a], fold_radix(n, false), true, scaled ? 1.0 / double(n) : 1.0);
   }
