@@ -53,8 +53,8 @@ enum {
   /* Operand split of the tensor-core products (Section II-A: float32 accuracy from several reduced-precision
      pieces whose products are accumulated).  Both use 3
      products of 11-bit pieces with fp32 accumulation and meet the same error bound.  Default: fp16 pieces (KDFT:
-     when every transformed n_a % 4 == 0, TF32 pieces otherwise); FFT axes of 512 points take TF32 pieces unless fp16
-     ones are insisted on. */
+     when every transformed n_a % 4 == 0, TF32 pieces otherwise); FFT axes of 512 points and axes 0 of 256 points
+     take TF32 pieces unless fp16 ones are insisted on. */
   DFT3D_SPLIT_FP16 = 4u,        /* insist on fp16 pieces (operands scaled by exact powers of two: KDFT from the largest
                                    input magnitude, FFT per line; half the tensor-core instructions of TF32);
                                    DFT3D_ERR_UNSUPPORTED for KDFT when a transformed n_a is not a multiple of 4 */
@@ -188,7 +188,7 @@ size_t dft3d_plan_workspace_bytes(dft3d_plan_t plan);
  * 2 * slices + 1 when the workspace holds only a half, a quarter or an eighth of a cube. */
 int dft3d_plan_launches(dft3d_plan_t plan);
 
-/* DFT3D_SPLIT_FP16 or DFT3D_SPLIT_TF32: the operand split the plan uses (FFT axes of 512 points: see the flags); 0 for
+/* DFT3D_SPLIT_FP16 or DFT3D_SPLIT_TF32: the operand split the plan uses (FFT axes of 256 and 512 points: see the flags); 0 for
  * NULL. */
 int dft3d_plan_split(dft3d_plan_t plan);
 

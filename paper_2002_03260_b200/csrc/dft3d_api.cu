@@ -818,6 +818,7 @@ int launch_fold(dft3d_plan_s* p, int a, const float* in, float* out, long long l
   fp.np = (2 * m + 15) / 16 * 16;
   fp.ks = ax.fold_t32 ? (2 * m + 7) / 8 : (2 * m + 15) / 16;
   fp.panels = (fp.ks + 3) / 4;
+  fp.twin = p->f16;
   fp.pre = ax.fold_pre;
   fp.in_scale = ax.fold_scale;
   fp.w_bytes = ax.fold_w_bytes;

@@ -50,6 +50,7 @@ struct FoldParams {
   unsigned C, off;          // STRIDED, natural order: line l starts at (l / C) * pitch + off + l % C, its points are `step` apart
   size_t pitch, step;
   int prefetch;             // L2 prefetch of later units
+  int twin;                 // TF32 pieces: two accumulators
   float pre, in_scale;      // TF32 pieces: factors before the R-point sums and on the phases (fp16: from amax_in)
   int in_blocked, out_blocked;   // columns per block, 0 = natural order: layouts of the intermediate between axes 0 and 1, see fold_place
   unsigned n0, n1, n2;      // the cube or the slice of its last axis (blocked layouts only)
@@ -392,7 +393,8 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
 
   // TF32 steps contract 8 instead of 16: twice as many additions that truncate.  Even and odd steps take accumulators of
   // their own (np <= 64 there), which the epilogue adds in round-to-nearest fp32.
-  const bool twin = T32 && p.ks >= 2;
+  // Only where fp16 pieces are what the axis would have otherwise: it costs up to 9 % (100 x 66 x 250: 36.8 -> 40.1 us).
+  const bool twin = T32 && p.twin && p.ks >= 2;
 
   if (warp < 4) {
     ptx::setmaxnreg_dec<40>();
