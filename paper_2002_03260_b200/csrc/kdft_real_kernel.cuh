@@ -314,9 +314,11 @@ kdft_real_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid
     const int m = q * 32 + lane;
     const int line = m >> 1, comp = m & 1;
     const float tau = comp ? 1.0f : -1.0f;   // i*w has the real part -Im w and the imaginary part Re w
-    // one factor where it is a normal number, else the two one after the other
+    // One factor where neither a sum (below 2^38) nor its share in the recombination can leave the normal numbers, else
+    // out_mul (2^-10 and the like) before the recombination and the scale of the data after it: a result that is a float
+    // is reached from either end of the range.
     const float both = p.out_mul * out_mul2;
-    const bool one_step = both > 1e-30f && both < 1e30f;
+    const bool one_step = both > 1e-26f && both < 1e26f;
     const float mul = one_step ? both : p.out_mul, taum = tau * mul;
     const int width = ((p.bn + 1) / 2 + 31) / 32 * 32;       // columns of the first of the two halves, at most 128
     const uint32_t lane_addr = tmem + (uint32_t(q * 32) << 16) + half * width;
@@ -353,10 +355,6 @@ kdft_real_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid
       // ---- undo the scales, recombine the lanes of a line, note the largest magnitude for the next pass, store
       float amax = 0.0f;
       if (ncols > 0) {
-        if (!one_step) {
-#pragma unroll
-          for (int i = 0; i < 128; ++i) acc[i] *= out_mul2;
-        }
         if (FORM == 1) {                       // columns (C_p, S_p) -> outputs N/2 + p and N/2 - 1 - p
           const float st = p.sign * taum;
 #pragma unroll
@@ -376,6 +374,10 @@ kdft_real_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid
             acc[2 * i] = fmaf(acc[2 * i] * mul, f.x, o0 * taum * f.y);
             acc[2 * i + 1] = fmaf(acc[2 * i + 1] * mul, f.z, o1 * taum * f.w);
           }
+        }
+        if (!one_step) {
+#pragma unroll
+          for (int i = 0; i < 128; ++i) acc[i] *= out_mul2;
         }
         long long base, step = 1;              // complex index of the line's first point, distance of its points
         bool live;

@@ -63,3 +63,45 @@ def test_solve_on_single_axes(lib, oracle, shape, axis, on_output):
     plan.destroy()
     want = oracle.solve_axis(x.cpu().numpy().astype(np.complex128), axis, nodes[axis], nodes_on_output=on_output)
     assert oracle.rel_l2(y.cpu().numpy(), want) < 2e-5
+
+
+def _one_axis(lib, x, axis, nodes, **kw):
+    plan = lib.Plan(*x.shape, nodes=nodes, axes=(axis,), **kw)
+    y = plan(x)
+    torch.cuda.synchronize()
+    plan.status()
+    plan.destroy()
+    return y
+
+
+# (axis, points, nodes): every form of the kernel; the uniform 260 points have no folded form
+RANGE_CASES = [(0, 64, "in"), (0, 64, "out"), (1, 64, "in"), (1, 64, "out"), (2, 64, "in"), (2, 64, "out"), (2, 260, "")]
+
+
+def _range_case(lib, axis, n, where):
+    shape = [4, 4, 4]
+    shape[axis] = n
+    nodes = [None] * 3
+    if where:
+        nodes[axis] = (np.arange(n) + np.random.default_rng(405).uniform(-0.3, 0.3, n)) / n
+    return shape, nodes, lib.DFT3D_NODES_ON_OUTPUT if where == "out" else 0
+
+
+@pytest.mark.parametrize("axis,n,where", RANGE_CASES)
+@pytest.mark.parametrize("sign,unscaled", [(-1, False), (+1, False), (+1, True)])
+@pytest.mark.parametrize("power", [100, 118, 123, 126, -100, -110])
+def test_single_samples_scale_like_any_other(lib, axis, n, where, sign, unscaled, power):
+    """A single sample spreads over its line with its own magnitude, so the result at 2^power is a normal number and
+    equals the scaled result bit for bit: every scale is a power of two, and no step may leave the float range."""
+    shape, nodes, flags = _range_case(lib, axis, n, where)
+    flags |= lib.DFT3D_UNSCALED_INVERSE if unscaled else 0
+    x = torch.zeros(shape, dtype=torch.complex64, device="cuda")
+    at = [1, 2, 3]
+    at[axis] = n // 3
+    x[tuple(at)] = 0.75 - 0.5j
+    y = _one_axis(lib, x, axis, nodes, sign=sign, flags=flags)
+    z = _one_axis(lib, x * 2.0 ** power, axis, nodes, sign=sign, flags=flags)
+    want = torch.view_as_real(y) * 2.0 ** power
+    normal = want.abs() >= 2.0 ** -126         # small components of the phases may be subnormal: they round once more
+    assert torch.equal(torch.view_as_real(z)[normal], want[normal])
+    assert (torch.view_as_real(z) - want).abs().max().item() <= (2.0 ** -149 if power < 0 else 0.0)
