@@ -443,7 +443,7 @@ int build_real_axis(dft3d_plan_s* p, KdftAxis& ax, const double* nodes, const do
     T.resize(size_t(n) * n);
     ph.resize(size_t(2) * n);
     H.assign(2 * piece, __float2half_rn(0.0f));
-    phf.assign(ax.form == 1 ? size_t(4) * ax.phase_pitch : size_t(2) * ((n + 255) / 256 * 256), 0.0f);
+    phf.assign(ax.form == 1 ? size_t(4) * dft3d::kRealPhaseSets * ax.phase_pitch : size_t(2) * ((n + 255) / 256 * 256), 0.0f);
   } catch (const std::bad_alloc&) {
     return fail(DFT3D_ERR_ALLOC, "host allocation of a real axis table failed");
   }
@@ -481,10 +481,14 @@ int build_real_axis(dft3d_plan_s* p, KdftAxis& ax, const double* nodes, const do
   for (long long j = 0; j < n; ++j) {
     const float re = float(ph[2 * j]), im = float(ph[2 * j + 1]);
     if (ax.form == 1) {                                   // z = re*a + im*b: (re, -im) for the real lane, (im, re) for the other
-      phf[2 * j] = re;
-      phf[2 * j + 1] = -im;
-      phf[2 * (ax.phase_pitch + j)] = im;
-      phf[2 * (ax.phase_pitch + j) + 1] = re;
+      for (int set = 0; set < dft3d::kRealPhaseSets; ++set) {
+        const float up = std::ldexp(1.0f, dft3d::real_phase_up(set));
+        float* to = &phf[2 * (size_t(2) * set * ax.phase_pitch + j)];
+        to[0] = up * re;
+        to[1] = up * -im;
+        to[2 * ax.phase_pitch] = up * im;
+        to[2 * ax.phase_pitch + 1] = up * re;
+      }
     } else {
       phf[2 * j] = re;
       phf[2 * j + 1] = im;

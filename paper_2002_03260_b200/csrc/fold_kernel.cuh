@@ -96,11 +96,6 @@ __host__ __device__ constexpr size_t fold_smem_bytes(unsigned w_bytes, int panel
 struct C2 {
   uint64_t re, im;
 };
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
 __device__ __forceinline__ uint64_t dup2(float a) { return pack2(a, a); }
 __device__ __forceinline__ C2 c2_add(C2 a, C2 b) { return {add2(a.re, b.re), add2(a.im, b.im)}; }
 __device__ __forceinline__ C2 c2_sub(C2 a, C2 b) { return {sub2(a.re, b.re), sub2(a.im, b.im)}; }

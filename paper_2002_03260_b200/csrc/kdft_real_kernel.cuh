@@ -32,12 +32,17 @@ constexpr int kRealPhaseBytes = 2 * 32 * 8;                // FORM 1: phases of 
 constexpr size_t kKdftRealSmemBytes =
     size_t(kRealStagesB) * kBytesStageB + size_t(kRealHalves) * (kRealBytesHalf + kRealPhaseBytes) + 1024 + 512;
 
+// FORM 1: the powers of two in the three sets of phases (ordinary data, data near the top and near the bottom of the range)
+constexpr int kRealPhaseSets = 3;
+__host__ __device__ constexpr int real_phase_up(int set) { return set == 1 ? -32 : (set == 2 ? 64 : 0); }
+
 struct KdftRealParams {
   int n, bn, n_tiles, chunk_kb;         // table columns per tile; chunk_kb counts 64-real stages
   long long m_tiles, rows, batches, C;
   int lpb, bpt;                         // lines of one batch in a tile, batches per tile
   long long c_tiles;
-  const float* phase;                   // FORM 1: [lane kind][n padded to 64] pairs (a, b): z = re*a + im*b; FORM 2: (re, im) per k
+  const float* phase;                   // FORM 1: [kRealPhaseSets][lane kind][n padded to 64] pairs (a, b): z = re*a + im*b;
+                                        // FORM 2: (re, im) per k
   int phase_pitch;                      // FORM 1: n padded to 64
   float sign;
   float* out;
@@ -120,15 +125,23 @@ kdft_real_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid
 
   // power-of-two scale that brings the largest input magnitude into [2^13, 2^14): fp16 pieces then neither
   // overflow nor lose more than fp16's own subnormal floor (2^-25 of a scaled unit) on small entries
-  float in_scale = 1.0f, out_mul2 = 1.0f;
+  // FORM 1 multiplies by the phase before it scales.  Data near either end of the float range takes phases that bring it
+  // towards the middle (`up`: powers of two, tables of their own), so that neither the two products overflow together
+  // nor their bits fall below the subnormal numbers.
+  float in_scale = 1.0f, out_mul1 = p.out_mul, out_mul2 = 1.0f;
+  const float* phase = p.phase;
   {
     const float a = __uint_as_float(*p.amax_in);
     if (a > 0.0f && a < 3.0e38f) {
-      // below 2^-113 the scale stops growing (2^126 is the largest power of two that is safe to multiply by);
-      // nothing is lost: such data are multiples of 2^-149, i.e. of 2^-23 after scaling, which the two pieces hold
-      const int e = max(ilogbf(a), -113);
-      in_scale = ldexpf(1.0f, 13 - e);
-      out_mul2 = ldexpf(1.0f, e - 13);
+      // FORM 2: below 2^-113 the scale stops growing (2^126 is the largest power of two that is safe to multiply by);
+      // nothing is lost: the sums of such data are multiples of 2^-149, i.e. of 2^-23 after scaling, which the two pieces hold
+      const int e = FORM == 1 ? ilogbf(a) : max(ilogbf(a), -113);
+      int up = 0;
+      if (FORM == 1 && e > 100) { up = real_phase_up(1); phase += 4 * p.phase_pitch; }
+      if (FORM == 1 && e < -60) { up = real_phase_up(2); phase += 8 * p.phase_pitch; }
+      in_scale = ldexpf(1.0f, 13 - e - up);
+      out_mul1 = ldexpf(p.out_mul, -up);
+      out_mul2 = ldexpf(1.0f, e - 13 + up);
     }
   }
 
@@ -175,7 +188,7 @@ kdft_real_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid
                 }
                 for (int c = 0; c < 2; ++c)
                   ptx::bulk_load(smem_ph + s * kRealPhaseBytes + c * (kRealPhaseBytes / 2),
-                                 p.phase + 2 * (size_t(c) * p.phase_pitch + j0), kRealPhaseBytes / 2, &sh.a_full[s]);
+                                 phase + 2 * (size_t(c) * p.phase_pitch + j0), kRealPhaseBytes / 2, &sh.a_full[s]);
               } else {                     // 16 pairs: the points left of the centre, then those right of it
                 const int p0 = kb * (kF16BlockK / 2) + 16 * h, left = p.n / 2 - 16 - p0, right = p.n / 2 + p0;
                 if (MODE == KDFT_CONTIG) {
@@ -242,8 +255,12 @@ kdft_real_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid
     const int line = m >> 1, comp = m & 1;
     // STRIDED: complex index of this lane's line in row 0 of a box (FORM 1: 32 rows per half, FORM 2: two boxes of 16)
     const int col = MODE == KDFT_STRIDED ? (line / p.lpb) * (FORM == 1 ? 32 : 16) * p.lpb + line % p.lpb : 0;
-    const float dsign = comp ? p.sign : -p.sign;      // FORM 2: s*i*d has the real part -s*Im d and the imaginary part s*Re d
-    const uint64_t scale2 = pack2(in_scale, FORM == 2 ? dsign * in_scale : in_scale);
+    // FORM 2: s*i*d has the real part -s*Im d and the imaginary part s*Re d.  The real lane takes (Re u, -s*Im d) from (re, im) of
+    // the two points, the imaginary lane (s*Re d, Im u).
+    const float ds = comp ? p.sign * in_scale : -p.sign * in_scale;
+    const uint64_t scale2 = FORM == 1 ? pack2(in_scale, in_scale) : (comp ? pack2(ds, in_scale) : pack2(in_scale, ds));
+    const uint64_t scale_l = comp ? pack2(-ds, in_scale) : pack2(in_scale, -ds);
+    const uint32_t order = comp ? 0x1032u : 0x3210u;
     uint32_t ia = 0, it = 0;
     for (long long t = blockIdx.x; t < total_tiles; t += gridDim.x) {
       for (int kb = 0; kb < num_kb; ++kb) {
@@ -273,16 +290,21 @@ kdft_real_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid
           } else {
 #pragma unroll
             for (int c = 0; c < 16; ++c) {         // pair c: point 15 - c of the left box, point c of the right one
-              const float *l, *r;
+              const uint8_t *l, *r;
               if (MODE == KDFT_CONTIG) {
                 const uint8_t* row = stage + line * 128;
-                l = reinterpret_cast<const float*>(row + ((((15 - c) >> 1) ^ (line & 7)) << 4) + ((15 - c) & 1) * 8);
-                r = reinterpret_cast<const float*>(row + kRealBytesHalf / 2 + (((c >> 1) ^ (line & 7)) << 4) + (c & 1) * 8);
+                l = row + ((((15 - c) >> 1) ^ (line & 7)) << 4) + ((15 - c) & 1) * 8;
+                r = row + kRealBytesHalf / 2 + (((c >> 1) ^ (line & 7)) << 4) + (c & 1) * 8;
               } else {
-                l = reinterpret_cast<const float*>(stage) + 2 * (col + (15 - c) * p.lpb);
-                r = reinterpret_cast<const float*>(stage + kRealBytesHalf / 2) + 2 * (col + c * p.lpb);
+                l = stage + 8 * (col + (15 - c) * p.lpb);
+                r = stage + kRealBytesHalf / 2 + 8 * (col + c * p.lpb);
               }
-              split_half2(mul2(pack2(r[comp] + l[comp], r[1 - comp] - l[1 - comp]), scale2), ph[h * 16 + c], pl[h * 16 + c]);
+              // (u, v), the other way round in the imaginary lane; scaled before they are added: a sum of two floats may be none.
+              // Whole points in one load each (nodes on the output, 256^3: 259 us; with 4-byte loads in the lane's order 276 us)
+              uint32_t hi, lo;
+              split_half2(fma2(*reinterpret_cast<const uint64_t*>(l), scale_l, mul2(*reinterpret_cast<const uint64_t*>(r), scale2)), hi, lo);
+              ph[h * 16 + c] = __byte_perm(hi, 0, order);
+              pl[h * 16 + c] = __byte_perm(lo, 0, order);
             }
           }
           // the half is refilled by TMA (async proxy): order this thread's reads before that write
@@ -315,11 +337,11 @@ kdft_real_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __grid
     const int line = m >> 1, comp = m & 1;
     const float tau = comp ? 1.0f : -1.0f;   // i*w has the real part -Im w and the imaginary part Re w
     // One factor where neither a sum (below 2^38) nor its share in the recombination can leave the normal numbers, else
-    // out_mul (2^-10 and the like) before the recombination and the scale of the data after it: a result that is a float
+    // the table's (2^-10 and the like) before the recombination and the scale of the data after it: a result that is a float
     // is reached from either end of the range.
-    const float both = p.out_mul * out_mul2;
+    const float both = out_mul1 * out_mul2;
     const bool one_step = both > 1e-26f && both < 1e26f;
-    const float mul = one_step ? both : p.out_mul, taum = tau * mul;
+    const float mul = one_step ? both : out_mul1, taum = tau * mul;
     const int width = ((p.bn + 1) / 2 + 31) / 32 * 32;       // columns of the first of the two halves, at most 128
     const uint32_t lane_addr = tmem + (uint32_t(q * 32) << 16) + half * width;
     const int chunks_per_tile = (num_kb + p.chunk_kb - 1) / p.chunk_kb;

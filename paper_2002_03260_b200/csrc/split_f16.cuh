@@ -30,6 +30,11 @@ __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
 
 // (re, im) -> packed fp16 pairs: hi = the value rounded to fp16, lo = the exact remainder x - hi rounded to fp16.
 __device__ __forceinline__ void split_half2(uint64_t x, uint32_t& hi, uint32_t& lo) {

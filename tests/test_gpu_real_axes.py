@@ -105,3 +105,38 @@ def test_single_samples_scale_like_any_other(lib, axis, n, where, sign, unscaled
     normal = want.abs() >= 2.0 ** -126         # small components of the phases may be subnormal: they round once more
     assert torch.equal(torch.view_as_real(z)[normal], want[normal])
     assert (torch.view_as_real(z) - want).abs().max().item() <= (2.0 ** -149 if power < 0 else 0.0)
+
+
+@pytest.mark.parametrize("axis,n,where", RANGE_CASES)
+@pytest.mark.parametrize("kind", ["inverse", "solve"])
+def test_samples_at_the_top_of_the_range(lib, axis, n, where, kind):
+    """Two samples that a pair sum adds, both components at 2.9e38: their sums and their products with the phases are no
+    floats, the results (scaled by 1/n, or a solve's) are, and equal those of the samples 2^-40 as large."""
+    if kind == "solve" and not where:
+        pytest.skip("a solve needs nodes")
+    shape, nodes, flags = _range_case(lib, axis, n, where)
+    flags |= lib.DFT3D_INVERSE_SOLVE if kind == "solve" else 0
+    x = torch.zeros(shape, dtype=torch.complex64, device="cuda")
+    for j in (n // 2 - 3, n // 2 + 2):
+        at = [1, 2, 3]
+        at[axis] = j
+        x[tuple(at)] = 2.9e38 + 2.9e38j
+    y = torch.view_as_real(_one_axis(lib, torch.view_as_complex(torch.view_as_real(x) * 2.0 ** -40), axis, nodes, sign=+1, flags=flags))
+    z = torch.view_as_real(_one_axis(lib, x, axis, nodes, sign=+1, flags=flags))
+    assert torch.equal(z, y * 2.0 ** 40) and bool(torch.isfinite(z).all())
+
+
+@pytest.mark.parametrize("axis,n,where", RANGE_CASES)
+@pytest.mark.parametrize("sign", [-1, +1])
+def test_subnormal_samples_lose_nothing_before_the_store(lib, axis, n, where, sign):
+    """Dense data of 2^-140, multiples of 2^-149 all: the results are what the same samples 2^120 as large give, rounded
+    to the grid of the subnormal numbers (half a step; one is asserted)."""
+    shape, nodes, flags = _range_case(lib, axis, n, where)
+    flags |= lib.DFT3D_UNSCALED_INVERSE if sign > 0 else 0
+    g = torch.Generator(device="cuda").manual_seed(406)
+    steps = torch.randint(-512, 513, shape + [2], generator=g, device="cuda").double()
+    big = torch.view_as_complex((steps * 2.0 ** -29).float())
+    small = torch.view_as_complex((steps * 2.0 ** -149).float())
+    y = torch.view_as_real(_one_axis(lib, big, axis, nodes, sign=sign, flags=flags)).double() * 2.0 ** -120
+    z = torch.view_as_real(_one_axis(lib, small, axis, nodes, sign=sign, flags=flags)).double()
+    assert (z - y).abs().max().item() <= 2.0 ** -149
