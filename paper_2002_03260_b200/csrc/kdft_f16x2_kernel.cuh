@@ -161,7 +161,7 @@ kdft_f16x2_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __gri
   float in_scale = 1.0f, out_mul2 = 1.0f;
   {
     const float a = __uint_as_float(*p.amax_in);
-    if (a > 0.0f && a < 3.0e38f) {
+    if (a > 0.0f) {                      // never an infinity: the reduction and the epilogues leave those out
       // below 2^-113 the scale stops growing (2^126 is the largest power of two that is safe to multiply by);
       // nothing is lost: such data are multiples of 2^-149, i.e. of 2^-23 after scaling, which the two pieces hold
       const int e = max(ilogbf(a), -113);

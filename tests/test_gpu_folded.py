@@ -141,3 +141,13 @@ def test_lines_beside_an_infinity_keep_their_values(lib):
     lost[1, 3] = lost[2, 5] = True
     assert not bool(torch.isfinite(torch.view_as_real(z[lost])).all())
     assert _rel(z[~lost], y[~lost]) < 1e-6         # the scale may differ by a power of two, the pieces with it
+
+
+@pytest.mark.parametrize("n", [64, 260, 2048])     # the folded, the real-matrix and the paired-CTA kernel
+def test_scaled_inverse_of_the_largest_floats(lib, n):
+    """The largest sample lies between 3.0e38 and the largest float: it is scaled like any other."""
+    x = torch.zeros((4, 4, n), dtype=torch.complex64, device="cuda")
+    x[1, 2, 5] = 3.2e38 - 1e37j
+    y = _run(lib, x, axes=(2,), sign=+1)
+    assert _rel(torch.view_as_complex(torch.view_as_real(y) * 2.0 ** -40),
+                torch.fft.ifft(x.to(torch.complex128), dim=2) * 2.0 ** -40) < BOUND
