@@ -832,7 +832,7 @@ int launch_fold(dft3d_plan_s* p, int a, const float* in, float* out, long long l
   fp.off = unsigned(n2_off);
   fp.pitch = size_t(n2_sub && a == 0 ? p->n[2] : ax.n * C);   // a slice of axis 0: one stretch of columns per i1
   fp.step = size_t(C);
-  fp.units = unsigned((lines + L - 1) / L);
+  fp.units = (fp.lines + unsigned(L) - 1) / unsigned(L);      // of the slice, where there is one
   fp.tasks = (unsigned(L) * fp.groups + 31) / 32;
   // see the kernel's loop over tasks: a unit of two tiles fills both buffers, a unit of one tile every other one
   const unsigned warps = H == 2 ? fp.tasks : 2 * fp.tasks;

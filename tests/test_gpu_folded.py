@@ -151,3 +151,29 @@ def test_scaled_inverse_of_the_largest_floats(lib, n):
     y = _run(lib, x, axes=(2,), sign=+1)
     assert _rel(torch.view_as_complex(torch.view_as_real(y) * 2.0 ** -40),
                 torch.fft.ifft(x.to(torch.complex128), dim=2) * 2.0 ** -40) < BOUND
+
+
+def test_slices_do_the_work_of_their_lines_only(lib):
+    """An eighth of a cube of workspace: the strided passes run once per slice, and each takes the time of its own lines.
+    (The same schedule with fp16 pieces has always done that; four times its time means whole-cube work per slice.)"""
+    shape = (256, 512, 512)
+    x = torch.zeros(shape, dtype=torch.complex64, device="cuda")
+    out = torch.empty_like(x)
+    took = []
+    for flags in (0, lib.DFT3D_SPLIT_FP16):
+        plan = lib.Plan(*shape, mode=lib.DFT3D_FFT, workspace_limit=1 << 26, flags=flags)
+        assert plan.launches == 17
+        for _ in range(3):
+            plan(x, out)
+        best = float("inf")
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            plan(x, out)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        plan.status()
+        plan.destroy()
+        took.append(best)
+    assert took[0] < 2.0 * took[1]
