@@ -412,6 +412,7 @@ kdft_f16x2_axis_kernel(const __grid_constant__ CUtensorMap map_data, const __gri
           }
         }
       }
+      amax = finite_magnitude(amax);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
       if (lane == 0 && amax > 0.0f) atomicMax(p.amax_out, __float_as_uint(amax));

@@ -177,3 +177,24 @@ def test_slices_do_the_work_of_their_lines_only(lib):
         plan.destroy()
         took.append(best)
     assert took[0] < 2.0 * took[1]
+
+
+@pytest.mark.parametrize("shape,axes", [((2, 2048, 8), (1, 2)), ((4, 4, 2048), (0, 2))])
+def test_an_overflow_in_a_paired_pass_spares_the_lines_beside_it(lib, shape, axes):
+    """A 2048-point pass (paired CTAs) before a shorter one: a line of 3e35 sums to an infinity at frequency zero, which
+    has no say in the second pass's scale; the lines that it does not reach keep their values."""
+    from paper_2002_03260_b200 import inputs
+    x = inputs.cube(shape, "normal", 307, device="cuda") * 1e30
+    y = _run(lib, x, axes=axes)
+    bad = x.clone()
+    keep = torch.ones(shape, dtype=torch.bool, device="cuda")
+    if 0 in axes:
+        bad[1, 3] = 3e35
+        keep[:, 3] = False                         # axis 0 spreads it over the planes
+    else:
+        bad[1, :, 5] = 3e35
+        keep[1] = False
+    z = _run(lib, bad, axes=axes)
+    assert not bool(torch.isfinite(torch.view_as_real(z[~keep])).all())
+    assert _rel(torch.view_as_complex(torch.view_as_real(z[keep]) * 2.0 ** -100),
+                torch.view_as_complex(torch.view_as_real(y[keep]) * 2.0 ** -100)) < 1e-6   # the scale may differ
