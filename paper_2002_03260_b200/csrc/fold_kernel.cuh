@@ -246,14 +246,15 @@ __device__ __forceinline__ void split_tf32(C2 x, uint32_t (&hi)[4], uint32_t (&l
   }
 }
 
-// Loads of the data, and explicit shared-memory accesses.  The 8-byte form takes whole lines per warp; of the 16-byte form a
+// Loads of the data (ordinary ones: a pass may run in place, and may start while its predecessor still writes), and explicit
+// shared-memory accesses.  The 8-byte form takes whole lines per warp; of the 16-byte form a
 // warp's lanes may be 32 bytes apart, and the second load finds the other halves of the sectors in L1 (512-point lines:
 // 582 us with, 620 us without).
 __device__ __forceinline__ void ld_stream8(const float2* p, float& a, float& b) {
-  asm volatile("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(a), "=f"(b) : "l"(p));
+  asm volatile("ld.global.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(a), "=f"(b) : "l"(p));
 }
 __device__ __forceinline__ void ld_stream16(const float2* p, float& a, float& b, float& c, float& d) {
-  asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
                : "=f"(a), "=f"(b), "=f"(c), "=f"(d) : "l"(p));
 }
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
