@@ -58,8 +58,9 @@ enum {
   DFT3D_SPLIT_FP16 = 4u,        /* insist on fp16 pieces (operands scaled by exact powers of two: KDFT from the largest
                                    input magnitude, FFT per line; half the tensor-core instructions of TF32);
                                    DFT3D_ERR_UNSUPPORTED for KDFT when a transformed n_a is not a multiple of 4 */
-  DFT3D_SPLIT_TF32 = 8u,        /* insist on TF32 pieces (no scaling; every element keeps ~22 significant bits
-                                   whatever the dynamic range of the input) */
+  DFT3D_SPLIT_TF32 = 8u,        /* insist on TF32 pieces (every element keeps ~22 significant bits whatever the dynamic
+                                   range of the input; no scaling, but for lines of an axis in folded form (see
+                                   dft3d_plan_create) whose largest component lies below 2^-96 or above 2^116) */
   DFT3D_DESTROY_INPUT = 16u,    /* dft3d_execute may overwrite `in`: a plan over all three axes then uses the input
                                    cube as its workspace and allocates none, which keeps the fast schedules available
                                    when input + output fill the memory (2048^3).  Ignored by plans over fewer axes. */

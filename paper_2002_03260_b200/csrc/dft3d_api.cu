@@ -181,7 +181,6 @@ struct KdftAxis {
   uint8_t* d_fold_w = nullptr;   // the m-point table as it lies in shared memory
   float4* d_fold_tw = nullptr;   // [fold_r][mp / 2] phases of pairs of points
   unsigned fold_w_bytes = 0;
-  float fold_pre = 1.0f, fold_scale = 1.0f;   // TF32 pieces: factors before the R-point sums and on the phases
 };
 
 struct FftAxis {
@@ -278,7 +277,7 @@ int fold_radix(long long n, bool f16) {
     if (!f16 && n % 4 != 0 && n % r == 0 && n / r <= 32) return r;
   return 0;
 }
-constexpr size_t kFoldSmemMax = dft3d::fold_smem_bytes(64 * 1024, 2, 1024);
+constexpr size_t kFoldSmemMax = dft3d::fold_smem_bytes(64 * 1024, 2, 1024, true);
 
 // the opt-in to large dynamic shared memory is a per-device property of each kernel
 int set_kernel_attributes(int device) {
@@ -412,13 +411,7 @@ int build_fold_axis(dft3d_plan_s* p, KdftAxis& ax, int r, bool t32, double scale
   ax.fold_r = r;
   ax.fold_w_bytes = unsigned(W.size());
   ax.fold_t32 = t32;
-  if (!t32) {
-    ax.out_mul = float(scale / 1024.0);
-  } else if (scale != 1.0) {
-    // TF32 pieces carry no scale that keeps large data in range, so the 1/n of a scaled inverse is taken before the sums
-    ax.fold_pre = 1.0f / float(r);
-    ax.fold_scale = 1.0f / float(m);
-  }
+  ax.out_mul = float(t32 ? scale : scale / 1024.0);
   DFT3D_CUDA(cudaMalloc(&ax.d_fold_w, W.size()));
   DFT3D_CUDA(cudaMemcpy(ax.d_fold_w, W.data(), W.size(), cudaMemcpyHostToDevice));
   DFT3D_CUDA(cudaMalloc(&ax.d_fold_tw, tw.size() * sizeof(float)));
@@ -823,8 +816,6 @@ int launch_fold(dft3d_plan_s* p, int a, const float* in, float* out, long long l
   fp.ks = ax.fold_t32 ? (2 * m + 7) / 8 : (2 * m + 15) / 16;
   fp.panels = (fp.ks + 3) / 4;
   fp.twin = p->f16;
-  fp.pre = ax.fold_pre;
-  fp.in_scale = ax.fold_scale;
   fp.w_bytes = ax.fold_w_bytes;
   fp.groups_magic = ((1u << 24) + fp.groups - 1) / fp.groups;
   fp.lines = unsigned(n2_sub ? lines / p->n[2] * n2_sub : lines);
@@ -834,6 +825,7 @@ int launch_fold(dft3d_plan_s* p, int a, const float* in, float* out, long long l
   fp.step = size_t(C);
   fp.units = (fp.lines + unsigned(L) - 1) / unsigned(L);      // of the slice, where there is one
   fp.tasks = (unsigned(L) * fp.groups + 31) / 32;
+  fp.block_tasks = L >= 32 ? fp.groups : fp.tasks;
   // see the kernel's loop over tasks: a unit of two tiles fills both buffers, a unit of one tile every other one
   const unsigned warps = H == 2 ? fp.tasks : 2 * fp.tasks;
   fp.split_warps = int(warps < unsigned(dft3d::kFoldSplitWarps) ? warps : unsigned(dft3d::kFoldSplitWarps));
@@ -851,7 +843,7 @@ int launch_fold(dft3d_plan_s* p, int a, const float* in, float* out, long long l
   fp.status = p->d_status;
   fp.wc = wait_control(p);
   const int grid = int(fp.units < unsigned(p->sm_count) ? fp.units : unsigned(p->sm_count));
-  const size_t smem = dft3d::fold_smem_bytes(fp.w_bytes, fp.panels, r * fp.mp);
+  const size_t smem = dft3d::fold_smem_bytes(fp.w_bytes, fp.panels, r * fp.mp, ax.fold_t32);
   const float sign = float(p->sign);
 #define DFT3D_FOLD_LAUNCH(MODE, R, T32)                                                                               \
   DFT3D_CUDA(launch_overlapped(p, dft3d::fold_axis_kernel<MODE, R, T32>, grid, dft3d::kFoldThreads, smem, stream, fp, sign))

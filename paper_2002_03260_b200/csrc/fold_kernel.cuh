@@ -29,6 +29,7 @@
 // coalesced as they are (16 or more neighbouring columns, or consecutive points of a line) and need no alignment beyond
 // a complex number's 8 bytes.
 #pragma once
+#include <type_traits>
 #include "kdft_f16_kernel.cuh"
 #include "split_f16.cuh"
 
@@ -51,12 +52,12 @@ struct FoldParams {
   size_t pitch, step;
   int prefetch;             // L2 prefetch of later units
   int twin;                 // TF32 pieces: two accumulators
-  float pre, in_scale;      // TF32 pieces: factors before the R-point sums and on the phases (fp16: from amax_in)
   int in_blocked, out_blocked;   // columns per block, 0 = natural order: layouts of the intermediate between axes 0 and 1, see fold_place
   unsigned n0, n1, n2;      // the cube or the slice of its last axis (blocked layouts only)
   unsigned units;           // groups of fold_lines lines
   unsigned tasks;           // warp-sized shares of a unit's loads and sums
-  int split_warps;          // warps that take them
+  unsigned block_tasks;     // TF32 pieces: the tasks that hold the groups of a line, block_tasks consecutive ones for up to 32 lines
+  int split_warps;          // warps that take the tasks
   float out_mul;
   const unsigned int* amax_in;
   unsigned int* amax_out;
@@ -69,6 +70,28 @@ struct FoldShared {
   uint32_t tmem_base;
   volatile int abort_flag;
   long long wait_limit;
+};
+
+// TF32 pieces need no scale unless a line lies near an end of the float range: with its largest component in [2^-96, 2^116) no
+// piece that matters is subnormal and no sum overflows.  Every task notes which of its lines have a component in that range and
+// which have one beyond; the epilogue passes over a unit that has a line with too large ones, or with too small ones only, and
+// the CTA takes these units once more when it is through with the others: then the tasks of a line wait for each other's
+// exponents and scale it to about 1.  (512-point axes 0 / 1 / 2 of 512^3: every line scaled that way 591 / 485 / 456 us, because
+// all warps wait for the slowest load of a unit; this way 479 / 444 / 416; no notes and no scale 496 / 444 / 401.)
+constexpr uint32_t kFoldLow = 127 - 96, kFoldHigh = 127 + 115;     // exponent fields
+constexpr unsigned kFoldTops = 8;        // units whose notes are kept: a warp that enters unit u has left u - 2 or a later one, whose
+                                         // buffer was free, so the product of u - 4 had been issued, the sums of u - 6 read
+constexpr unsigned kFoldMarks = 1 << 16; // units that a CTA can pass over; with more all take the second form
+struct FoldRange {
+  uint64_t top_full[kFoldTops][4];       // second form, per block of 32 lines: the exponents are complete
+  uint64_t split_done, first_done;       // every unit has been split once; has been stored or marked
+  // Words of a unit carry its position in the order of work plus one, so that an older one never counts.
+  uint32_t top[kFoldTops * 128];          // << 8 | 0: the line has a component in the range; second form: largest exponent field
+  uint32_t far[kFoldTops * 128];          // << 1 | 1: the line has a component above the range, | 0: one below (and not zero)
+  volatile uint32_t any_far[kFoldTops];
+  volatile uint32_t marks[kFoldMarks / 32];
+  volatile uint32_t marked;
+  volatile uint32_t far_seen;            // 0: nothing to take once more, no role waits for the others at its end
 };
 
 constexpr int kFoldThreads = 640;
@@ -87,8 +110,9 @@ __host__ __device__ constexpr int fold_lines(bool strided, int R) {
   return l;
 }
 constexpr int kFoldPanelBytes = 128 * 128;      // 128 lanes x 128 bytes
-__host__ __device__ constexpr size_t fold_smem_bytes(unsigned w_bytes, int panels, int tw_entries) {
-  return size_t(w_bytes) + size_t(4) * panels * kFoldPanelBytes + size_t(tw_entries) * 12 + sizeof(FoldShared) + 1024;
+__host__ __device__ constexpr size_t fold_smem_bytes(unsigned w_bytes, int panels, int tw_entries, bool t32) {
+  return size_t(w_bytes) + size_t(4) * panels * kFoldPanelBytes + size_t(tw_entries) * 12 + sizeof(FoldShared) +
+         (t32 ? sizeof(FoldRange) : 0) + 1024;
 }
 
 // ---- Two complex numbers at a time: re and im hold the real and the imaginary parts of two neighbouring points, so that
@@ -233,6 +257,28 @@ __device__ __forceinline__ void split_half2_scaled(C2 x, uint32_t& hi0, uint32_t
   lo1 = *reinterpret_cast<const uint32_t*>(&l1);
 }
 
+__device__ __forceinline__ float max_abs3(float a, float b, float c) {
+  float r;
+  asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+// Exponent fields as FoldRange holds them.  A line with an infinity (255) has no finite result at any scale.
+__device__ __forceinline__ uint32_t fold_field(float top) { return top > 0.0f ? max(__float_as_uint(top) >> 23, 1u) : 0; }
+__device__ __forceinline__ bool fold_outside(uint32_t f) { return f != 0 && f != 255 && (f < kFoldLow || f > kFoldHigh); }
+__device__ __forceinline__ int fold_shift(uint32_t f) { return f == 0 || f == 255 ? 0 : max(127 - int(f), -100); }
+__device__ __forceinline__ float pow2f(int e) { return __uint_as_float(uint32_t(127 + e) << 23); }
+// the first marked unit from `from` on, or `units`
+__device__ __forceinline__ unsigned fold_next(const FoldRange& rg, bool all, unsigned from, unsigned units) {
+  if (all || from >= units) return min(from, units);
+  unsigned w = from >> 5;
+  uint32_t b = rg.marks[w] & (0xffffffffu << (from & 31));
+  while (b == 0) {
+    if (++w * 32 >= units) return units;
+    b = rg.marks[w];
+  }
+  return w * 32 + __ffs(b) - 1;
+}
+
 // Two complex numbers -> TF32 pieces (re, im, re', im'): hi is the raw word (the tensor core ignores the low 13 bits of the
 // mantissa), lo the remainder rounded to TF32.
 __device__ __forceinline__ void split_tf32(C2 x, uint32_t (&hi)[4], uint32_t (&lo)[4]) {
@@ -297,14 +343,15 @@ __device__ __forceinline__ LinePlace fold_place(const FoldParams& p, unsigned l,
     atomicCAS(p.status, 0u, (unsigned)(code));                                         \
     goto role_done;                                                                    \
   }
-#define FOLD_WAIT_WARP(bar, parity, code)                                                                 \
+#define FOLD_WAIT_WARP_ELSE(bar, parity, code, leave)                                                     \
   if (!__all_sync(0xffffffffu, bounded_wait((bar), (parity), &sh.abort_flag, sh.wait_limit) ? 1 : 0)) {   \
     sh.abort_flag = 1;                                                                                    \
     atomicCAS(p.status, 0u, (unsigned)(code));                                                            \
-    goto role_done;                                                                                       \
+    leave;                                                                                                \
   }
+#define FOLD_WAIT_WARP(bar, parity, code) FOLD_WAIT_WARP_ELSE(bar, parity, code, goto role_done)
 
-// T32: TF32 pieces instead of fp16 ones (no scaling; twice the bytes per operand, so m <= 32)
+// T32: TF32 pieces instead of fp16 ones (twice the bytes per operand, so m <= 32; scales as FoldRange says)
 template <int MODE, int R, bool T32>
 __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldParams p, const float sign) {
   constexpr int H = fold_tiles(MODE == KDFT_STRIDED, R);   // tiles per unit
@@ -326,7 +373,14 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
   float4* smem_t = reinterpret_cast<float4*>(smem_a + 4 * size_t(piece_bytes));
   float2* smem_tn = reinterpret_cast<float2*>(smem_t + t_entries);
   FoldShared& sh = *reinterpret_cast<FoldShared*>(smem_tn + t_entries);
+  FoldRange& rg = *reinterpret_cast<FoldRange*>(&sh + 1);                   // TF32 pieces only
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+  // this CTA's units: blockIdx.x, blockIdx.x + gridDim.x, ...
+  const unsigned my_units = blockIdx.x < p.units ? (p.units - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+  // Positions in the order of work: first the units one by one, then (TF32 pieces) those that the epilogue marked.
+  const bool all = T32 && my_units > kFoldMarks;
+  const unsigned first = all ? 0 : my_units;
 
   ptx::griddep_launch();
   if (tid == 0) {
@@ -335,6 +389,12 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
       ptx::mbar_init(&sh.a_empty[i], 1);
       ptx::mbar_init(&sh.d_full[i], 1);
       ptx::mbar_init(&sh.d_empty[i], 4);
+    }
+    if (T32) {
+      ptx::mbar_init(&rg.split_done, unsigned(p.split_warps));
+      ptx::mbar_init(&rg.first_done, 4);
+      rg.marked = 0;
+      rg.far_seen = all;
     }
     ptx::mbar_init(&sh.w_full, 1);
     sh.abort_flag = 0;
@@ -355,8 +415,11 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
   // first so that the sums cannot overflow.
   float in_scale = 1.0f, out_mul2 = 1.0f, pre = 1.0f;
   if (T32) {
-    in_scale = p.in_scale;
-    pre = p.pre;
+    if (tid < 4 * kFoldTops) ptx::mbar_init(&rg.top_full[0][0] + tid, p.block_tasks);
+    if (tid < kFoldTops) rg.any_far[tid] = 0;
+    for (uint32_t i = tid; i < kFoldTops * L; i += kFoldThreads) rg.top[i] = rg.far[i] = 0;
+    if (!all)
+      for (uint32_t i = tid; i < (my_units + 31) / 32; i += kFoldThreads) rg.marks[i] = 0;
   } else {
     const float a = __uint_as_float(*p.amax_in);
     if (a > 0.0f) {                      // never an infinity: the reduction and the epilogues leave those out
@@ -383,17 +446,13 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
   ptx::tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
 
-  // this CTA's units: blockIdx.x, blockIdx.x + gridDim.x, ...
-  const unsigned my_units = blockIdx.x < p.units ? (p.units - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-  const unsigned my_tiles = my_units * H;
-
   // TF32 steps contract 8 instead of 16: twice as many additions that truncate.  Even and odd steps take accumulators of
   // their own (np <= 64 there), which the epilogue adds in round-to-nearest fp32.
   // Only where fp16 pieces are what the axis would have otherwise: it costs up to 9 % (100 x 66 x 250: 36.8 -> 40.1 us).
   const bool twin = T32 && p.twin && p.ks >= 2;
 
   if (warp < 4) {
-    ptx::setmaxnreg_dec<40>();
+    ptx::setmaxnreg_dec<32>();
     if (warp == 0 && lane == 0) {
       // ------------------------------------------------------------ MMA issuer
       const uint32_t idesc = T32 ? ptx::make_idesc_tf32(128, p.np) : ptx::make_idesc_f16(128, p.np);
@@ -402,7 +461,15 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
       const uint64_t a0 = ptx::make_kmajor_sw128_desc(ptx::smem_u32(smem_a));
       const uint32_t w_panel = uint32_t(2 * p.np * 128) >> 4;     // in descriptor address units
       FOLD_WAIT(&sh.w_full, 0, 0x701);
-      for (unsigned k = 0; k < my_tiles; ++k) {
+      unsigned tiles = first * H;
+      for (unsigned k = 0;; ++k) {
+        if (k == tiles) {
+          if (!T32 || tiles != first * H) break;
+          if (!rg.far_seen) break;
+          FOLD_WAIT(&rg.first_done, 0, 0x707);
+          tiles += (all ? my_units : rg.marked) * H;
+          if (k == tiles) break;
+        }
         const uint32_t buf = k & 1, ph = (k >> 1) & 1;
         FOLD_WAIT(&sh.d_empty[buf], ph ^ 1, 0x703);
         FOLD_WAIT(&sh.a_full[buf], ph, 0x702);
@@ -427,7 +494,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
     }
   } else if (warp < 8) {
     // -------------------------------------------------------------- epilogue
-    ptx::setmaxnreg_inc<104>();
+    ptx::setmaxnreg_inc<112>();
     const int row = (warp & 3) * 32 + lane;
     const uint32_t lane_addr = tmem + (uint32_t((warp & 3) * 32) << 16);
     const int q = MODE == KDFT_CONTIG ? row % Q : row / L;
@@ -438,9 +505,11 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
     const bool one_step = both > 1e-30f && both < 1e30f;
     const uint64_t mul_a = dup2(one_step ? both : p.out_mul), mul_b = dup2(out_mul2);
     float amax = 0.0f;
-    for (unsigned k = 0; k < my_tiles; ++k) {
+    // tile k in the order of work, of unit `unit`; false: a wait gave up
+    auto drain = [&](auto again, unsigned k, unsigned unit) -> bool {
+      constexpr bool kSecond = decltype(again)::value;
       const uint32_t buf = k & 1, ph = (k >> 1) & 1;
-      const unsigned l = (blockIdx.x + (k / H) * gridDim.x) * L + line;
+      const unsigned l = (blockIdx.x + unit * gridDim.x) * L + line;
       const bool live = l < p.lines && (MODE == KDFT_CONTIG ? line < unsigned(L) : q < Q);   // not an idle lane
       float2* dst;
       size_t step;
@@ -452,8 +521,24 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
         dst = p.out + at.base + (q + (k % H) * Q) * at.step;
         step = at.step * R;
       }
-      FOLD_WAIT_WARP(&sh.d_full[buf], ph, 0x704);
+      FOLD_WAIT_WARP_ELSE(&sh.d_full[buf], ph, 0x704, return false);
       ptx::tc_fence_after();
+      int shift = 0;
+      bool pass_over = false;
+      if (T32) {
+        const unsigned slot = k / H % kFoldTops, tag = k / H + 1;
+        const volatile uint32_t *top = rg.top + slot * L, *far = rg.far + slot * L;
+        if (kSecond) {
+          if (live) shift = fold_shift(top[line] & 0xff);
+        } else if (rg.any_far[slot] == tag) {
+          for (int i = lane; i < L; i += 32) pass_over |= far[i] >> 1 == tag && ((far[i] & 1) || top[i] >> 8 != tag);
+          pass_over = __any_sync(0xffffffffu, pass_over);
+          if (pass_over && k % H == H - 1 && warp == 4 && lane == 0) {
+            rg.marks[unit >> 5] = rg.marks[unit >> 5] | 1u << (unit & 31);
+            rg.marked = rg.marked + 1;
+          }
+        }
+      }
       for (int c0 = 0; c0 < 2 * p.m; c0 += 32) {
         uint32_t hh[32], xx[32];
         ptx::tmem_ld_32x32(lane_addr + buf * 256 + c0, hh);
@@ -479,13 +564,14 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
 #pragma unroll
         for (int i = 0; i < 16; ++i)
           v[i] = mul2(fma2(pack2_bits(xx[2 * i], xx[2 * i + 1]), down11, pack2_bits(hh[2 * i], hh[2 * i + 1])), mul_a);
-        if (!one_step) {
+        if (T32 ? kSecond && shift != 0 : !one_step) {
+          const uint64_t f = T32 ? dup2(pow2f(-shift)) : mul_b;
 #pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] = mul2(v[i], mul_b);
+          for (int i = 0; i < 16; ++i) v[i] = mul2(v[i], f);
         }
-        const int count = live ? p.m - c0 / 2 : 0;       // outputs of this line among the sixteen
+        const int count = live && !pass_over ? p.m - c0 / 2 : 0;       // outputs of this line among the sixteen
         float top = 0.0f;
-        if (count >= 16) {
+        if (!kSecond && count >= 16) {
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             float re, im;
@@ -507,6 +593,18 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
         }
         amax = fmaxf(amax, finite_magnitude(top));       // a line with an infinity has no say in the next pass's scale
       }
+      return true;
+    };
+    unsigned k = 0;
+    for (; k < first * H; ++k)
+      if (!drain(std::false_type(), k, k / H)) goto role_done;
+    if (T32 && __builtin_expect(rg.far_seen != 0, 0)) {
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(&rg.first_done);
+      FOLD_WAIT_WARP(&rg.first_done, 0, 0x707);
+      for (unsigned unit = fold_next(rg, all, 0, my_units); unit < my_units; unit = fold_next(rg, all, unit + 1, my_units))
+        for (int h = 0; h < H; ++h, ++k)
+          if (!drain(std::true_type(), k, unit)) goto role_done;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
@@ -520,10 +618,10 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
     // The tasks of all units go round the warps.  The host picks the number of warps such that no warp is so far ahead of
     // the buffers that the parity of a_empty could mean an older phase: consecutive units of a warp are neighbours, or
     // at most two apart where a unit uses one of the two buffers.
-    unsigned k = 0, j = unsigned(warp - 8);
-    while (true) {
-      while (j >= p.tasks) { j -= p.tasks; ++k; }
-      if (k >= my_units) break;
+    // Task j of unit `unit`, the k-th in the order of work; false: a wait gave up.  (Two copies of the code: one that also waits for the
+    // lines' exponents took 63 instead of 56 us on 256-point axes 0 of 256^3.)
+    auto split = [&](auto again, unsigned k, unsigned j, unsigned unit) -> bool {
+      constexpr bool kSecond = decltype(again)::value;
       const uint32_t buf = H == 2 ? 0 : k & 1, ph = (H == 2 ? k : k >> 1) & 1;
       unsigned line, grp;
       if (MODE == KDFT_CONTIG) {
@@ -532,14 +630,19 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
         grp = id - line * p.groups;
       } else {
         // sixteen lines: eight of them and two groups per half warp, so that its 8-byte operand stores meet every bank once
-        constexpr unsigned kWarps = L > 32 ? L / 32 : 1;           // warps side by side
-        line = L == 16 ? (lane & 7) | ((lane >> 4) << 3) : (j % kWarps) * 32 + lane;
-        grp = L == 16 ? j * 2 + ((lane >> 3) & 1) : j / kWarps;
+        // more than 32 lines: block by block
+        line = L == 16 ? (lane & 7) | ((lane >> 4) << 3) : lane;
+        grp = L == 16 ? j * 2 + ((lane >> 3) & 1) : j;
+        if (L > 32) {
+          const unsigned block = unsigned((uint64_t(j) * p.groups_magic) >> 24);
+          line += block * 32;
+          grp -= block * p.groups;
+        }
       }
       const bool mine = line < unsigned(L) && grp < p.groups;
       C2 x[B / 2][R];
       {
-        const unsigned l = (blockIdx.x + k * gridDim.x) * L + line;
+        const unsigned l = (blockIdx.x + unit * gridDim.x) * L + line;
         const float2* src;
         size_t C = 1;                                              // distance of neighbouring points of a line
         if (MODE == KDFT_CONTIG) {
@@ -551,7 +654,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
         }
         const size_t sstep = size_t(p.m) * C;
         const bool live = mine && l < p.lines;
-        if (live && (grp + 1) * B <= unsigned(p.m)) {
+        if (!kSecond && live && (grp + 1) * B <= unsigned(p.m)) {
           if (MODE == KDFT_CONTIG && wide) {
 #pragma unroll
             for (int s = 0; s < R; ++s, src += sstep)
@@ -587,8 +690,8 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
         }
       }
       // bring a later unit of this CTA into L2 meanwhile
-      if (p.prefetch && k + kAhead < my_units) {
-        const unsigned l0 = (blockIdx.x + (k + kAhead) * gridDim.x) * L;
+      if (p.prefetch && !kSecond && unit + kAhead < my_units) {
+        const unsigned l0 = (blockIdx.x + (unit + kAhead) * gridDim.x) * L;
         if (l0 < p.lines) {
           if (MODE == KDFT_CONTIG) {
             const char* base = reinterpret_cast<const char*>(p.in + size_t(l0) * p.n);
@@ -606,11 +709,47 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
           }
         }
       }
-      if (pre != 1.0f) {
+      float factor = pre;
+      if (T32) {                                                   // this task's share of its lines' exponents
+        float top = 0.0f;
 #pragma unroll
         for (int b = 0; b < B / 2; ++b)
 #pragma unroll
-          for (int s = 0; s < R; ++s) x[b][s] = {mul2(x[b][s].re, dup2(pre)), mul2(x[b][s].im, dup2(pre))};
+          for (int s = 0; s < R; ++s) {
+            float v0, v1, v2, v3;
+            unpack2(x[b][s].re, v0, v2);
+            unpack2(x[b][s].im, v1, v3);
+            top = max_abs3(max_abs3(top, v0, v1), v2, v3);
+          }
+        const unsigned slot = k % kFoldTops, tag = k + 1;
+        const uint32_t field = fold_field(top);
+        const uint32_t at = slot * L + (mine ? line : 0);
+        uint32_t* word = &rg.top[at];
+        if (!kSecond) {
+          if (mine && field != 0) {
+            if (!fold_outside(field)) {
+              *const_cast<volatile uint32_t*>(word) = tag << 8;
+            } else {
+              atomicMax(&rg.far[at], tag << 1 | (field > kFoldHigh));
+              rg.any_far[slot] = tag;
+              rg.far_seen = 1;
+            }
+          }
+        } else {
+          if (mine) atomicMax(word, tag << 8 | field);
+          const unsigned i = k - first, block = L > 32 ? unsigned((uint64_t(j) * p.groups_magic) >> 24) : 0;
+          uint64_t* bar = &rg.top_full[i % kFoldTops][block];
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(bar);
+          FOLD_WAIT_WARP_ELSE(bar, (i / kFoldTops) & 1, 0x706, return false);
+          factor = pow2f(mine ? fold_shift(*const_cast<volatile uint32_t*>(word) & 0xff) : 0);
+        }
+      }
+      if (T32 ? kSecond : factor != 1.0f) {
+#pragma unroll
+        for (int b = 0; b < B / 2; ++b)
+#pragma unroll
+          for (int s = 0; s < R; ++s) x[b][s] = {mul2(x[b][s].re, dup2(factor)), mul2(x[b][s].im, dup2(factor))};
       }
       {
         const uint32_t col = grp * (B * (T32 ? 8 : 4));            // bytes along the contraction
@@ -627,7 +766,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
         }
 #pragma unroll
         for (int h = 0; h < H; ++h) {
-          FOLD_WAIT_WARP(&sh.a_empty[buf + h], ph ^ 1, 0x705);
+          FOLD_WAIT_WARP_ELSE(&sh.a_empty[buf + h], ph ^ 1, 0x705, return false);
           if (mine) {
 #pragma unroll
             for (int q = h * Q; q < (h + 1) * Q; ++q) {
@@ -638,10 +777,10 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
 #pragma unroll
               for (int b = 0; b < B / 2; ++b) {
                 uint64_t c, d, dn;
-                lds_2x64(t_at + (uint32_t(q) * p.mp / 2 + b) * 16, c, d);
-                C2 u;
-                if (q == 0) {
-                  u = {mul2(x[b][0].re, c), mul2(x[b][0].im, c)};
+                C2 u = x[b][0];
+                if (!T32 || q != 0) lds_2x64(t_at + (uint32_t(q) * p.mp / 2 + b) * 16, c, d);
+                if (q == 0) {                  // the phases are 1, times the scale that the fp16 pieces need
+                  if (!T32) u = {mul2(u.re, c), mul2(u.im, c)};
                 } else {
                   lds_64(tn_at + (uint32_t(q) * p.mp / 2 + b) * 8, dn);
                   u = c2_mul(x[b][q], c, d, dn);
@@ -671,7 +810,31 @@ __global__ void __launch_bounds__(kFoldThreads, 1) fold_axis_kernel(const FoldPa
           if (lane == 0) ptx::mbar_arrive(&sh.a_full[buf + h]);
         }
       }
-      j += unsigned(p.split_warps);
+      return true;
+    };
+    unsigned k = 0, j = unsigned(warp - 8);
+    for (; j >= p.tasks; ++k) j -= p.tasks;
+    while (k < first) {
+      if (!split(std::false_type(), k, j, k)) goto role_done;
+      for (j += unsigned(p.split_warps); j >= p.tasks; ++k) j -= p.tasks;
+    }
+    if constexpr (T32) {
+      // far_seen is final when every warp has split its share
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(&rg.split_done);
+      FOLD_WAIT_WARP(&rg.split_done, 0, 0x708);
+      if (__builtin_expect(rg.far_seen != 0, 0)) {
+        FOLD_WAIT_WARP(&rg.first_done, 0, 0x707);
+        unsigned unit = fold_next(rg, all, 0, my_units);
+        for (unsigned i = first; i < k; ++i) unit = fold_next(rg, all, unit + 1, my_units);
+        while (unit < my_units) {
+          if (!split(std::true_type(), k, j, unit)) goto role_done;
+          for (j += unsigned(p.split_warps); j >= p.tasks; ++k) {
+            j -= p.tasks;
+            unit = fold_next(rg, all, unit + 1, my_units);
+          }
+        }
+      }
     }
   }
 
@@ -688,5 +851,6 @@ role_done:
 
 #undef FOLD_WAIT
 #undef FOLD_WAIT_WARP
+#undef FOLD_WAIT_WARP_ELSE
 
 }  // namespace dft3d

@@ -198,3 +198,85 @@ def test_an_overflow_in_a_paired_pass_spares_the_lines_beside_it(lib, shape, axe
     assert not bool(torch.isfinite(torch.view_as_real(z[~keep])).all())
     assert _rel(torch.view_as_complex(torch.view_as_real(z[keep]) * 2.0 ** -100),
                 torch.view_as_complex(torch.view_as_real(y[keep]) * 2.0 ** -100)) < 1e-6   # the scale may differ
+
+
+# ------------------------------------------------------------------ TF32 pieces: the ends of the float range, and the pieces
+
+# every R, contiguous and strided, in the formulation and with the pieces that choose it; "" leaves the pieces open
+RANGE_AXES = [("fft", "", 0, 256), ("fft", "", 0, 512), ("fft", "", 1, 512), ("fft", "", 2, 512), ("fft", "tf32", 1, 256),
+              ("fft", "tf32", 2, 256), ("fft", "tf32", 2, 512), ("kdft", "tf32", 1, 100), ("kdft", "tf32", 2, 100)]
+RANGE_AXES += [("kdft", "", a, n) for a in (1, 2) for n in (30, 62, 66, 150, 186, 250)]
+
+
+@pytest.mark.parametrize("mode,pieces,axis,n", RANGE_AXES)
+@pytest.mark.parametrize("sign", [-1, +1])
+@pytest.mark.parametrize("low,high", [(-120, 60), (-146, 124), (0, 0)])
+def test_every_line_keeps_its_precision_at_any_magnitude(lib, mode, pieces, axis, n, sign, low, high):
+    """Lines whose magnitudes differ by any power of two, side by side: each comes out with an error of 1e-6 of its own norm,
+    or half a step of the subnormal numbers per component."""
+    from paper_2002_03260_b200 import inputs
+    shape = [64, 64, 64] if mode == "fft" else [10, 34, 18]
+    shape[axis] = n
+    x = inputs.cube(tuple(shape), "uniform", 308, device="cuda")
+    g = torch.Generator(device="cuda").manual_seed(309)
+    lines = [1 if d == axis else shape[d] for d in range(3)]
+    power = torch.randint(low, high + 1, lines, generator=g, device="cuda").double()
+    if sign < 0:
+        power[power > 60] -= n.bit_length()        # the sums of n samples are floats
+    xs = torch.view_as_complex((torch.view_as_real(x).double() * torch.exp2(power)[..., None]).float())
+    y = _run(lib, xs, mode=lib.DFT3D_FFT if mode == "fft" else lib.DFT3D_KDFT, axes=(axis,), sign=sign,
+             flags=lib.DFT3D_SPLIT_TF32 if pieces else 0).to(torch.complex128)
+    want = (torch.fft.fft if sign < 0 else torch.fft.ifft)(xs.to(torch.complex128), dim=axis)
+    error = torch.linalg.vector_norm(y - want, dim=axis)
+    assert bool((error <= BOUND * torch.linalg.vector_norm(want, dim=axis) + 2.0 ** -149 * np.sqrt(n)).all())
+
+
+@pytest.mark.parametrize("pieces", ["", "tf32"])
+@pytest.mark.parametrize("limit", [0, 1 << 28, 1])
+@pytest.mark.parametrize("power", [-104, 100])
+def test_whole_cubes_near_the_ends_of_the_range(lib, pieces, limit, power):
+    """Lines of every pass that are taken twice, out of place, in slices and in place: bit for bit the scaled result."""
+    from paper_2002_03260_b200 import inputs
+    x = inputs.cube((512, 256, 512), "uniform", 310, device="cuda")
+    kw = dict(mode=lib.DFT3D_FFT, sign=+1, flags=(lib.DFT3D_SPLIT_TF32 if pieces else 0) | lib.DFT3D_UNSCALED_INVERSE,
+              workspace_limit=limit)
+    x[:, :, ::3] = 0                               # samples and lines of zeros among them
+    y = torch.view_as_real(_run(lib, x, **kw))
+    z = torch.view_as_real(_run(lib, torch.view_as_complex(torch.view_as_real(x) * 2.0 ** power), **kw))
+    want = y * 2.0 ** power
+    normal = want.abs() >= 2.0 ** -126
+    assert torch.equal(z[normal], want[normal]) and bool(((z - want)[~normal].abs() <= 2.0 ** -148).all())
+
+
+def test_more_units_than_a_block_can_mark(lib):
+    """3.2e8 lines of four points: with more than 65536 units a block scales every line by its own largest component."""
+    n0, n1 = 40000, 8000
+    x = torch.zeros((n0, n1, 4), dtype=torch.complex64, device="cuda")
+    g = torch.Generator(device="cuda").manual_seed(312)
+    rows = [0, 1, 19999, n0 - 1]
+    for i, r in enumerate(rows):
+        x[r] = torch.view_as_complex(torch.randn((n1, 4, 2), generator=g, device="cuda") * 2.0 ** (0, -110, 120, 3)[i])
+    y = _run(lib, x, axes=(2,), flags=lib.DFT3D_SPLIT_TF32)
+    for r in rows:
+        want = torch.fft.fft(x[r].to(torch.complex128), dim=1)
+        assert _rel(y[r].to(torch.complex128), want) < BOUND
+        y[r] = 0
+    assert not bool(torch.view_as_real(y).any())
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_lines_beside_infinities_with_tf32_pieces(lib, axis):
+    from paper_2002_03260_b200 import inputs
+    shape = [64, 64, 64]
+    shape[axis] = 512
+    x = inputs.cube(tuple(shape), "normal", 313, device="cuda")
+    y = _run(lib, x, mode=lib.DFT3D_FFT, axes=(axis,))
+    bad = x.clone()
+    bad[1, 3, 7] = complex(float("inf"), 0.0)
+    bad[2, 5, 9] = complex(0.0, float("nan"))
+    z = _run(lib, bad, mode=lib.DFT3D_FFT, axes=(axis,))
+    lost = torch.zeros(shape, dtype=torch.bool, device="cuda")
+    for at in ([1, 3, 7], [2, 5, 9]):
+        at[axis] = slice(None)
+        lost[tuple(at)] = True
+    assert not bool(torch.isfinite(z[lost]).any()) and torch.equal(z[~lost], y[~lost])
