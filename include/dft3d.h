@@ -77,12 +77,14 @@ typedef struct dft3d_options_s {
   size_t struct_size;     /* sizeof(dft3d_options_t), for forward compatibility */
   unsigned flags;         /* DFT3D_NODES_ON_OUTPUT | DFT3D_UNSCALED_INVERSE | DFT3D_SPLIT_* | DFT3D_DESTROY_INPUT */
   int fft_split[3][2];    /* FFT mode: {N1, N2} per axis with N1*N2 = n_a, first and second matrix product of Eq. 17.
-                             {0,0} = the built-in split, which is also the only one the kernels realise: N2 = 16 for
-                             n_a = 256 and 512, N2 = 32 from 1024 on, N1 = n_a / N2 (256 = 16*16, 512 = 32*16,
-                             1024 = 32*32, 2048 = 64*32, 4096 = 128*32; an N1 above N2 is itself computed as
-                             (N1/N2) * N2 by one more application of Eq. 17; 8192 = 1024*8, the 1024 again 32*32).
-                             Any other pair returns
-                             DFT3D_ERR_UNSUPPORTED; dft3d_plan_fft_split reports the pair in use. */
+                             {0,0} = the library's choice.  The pairs that can be named: N2 = 16 for n_a = 256 and
+                             512, N2 = 32 from 1024 on, N1 = n_a / N2 (256 = 16*16, 512 = 32*16, 1024 = 32*32,
+                             2048 = 64*32, 4096 = 128*32; an N1 above N2 is itself computed as (N1/N2) * N2 by one
+                             more application of Eq. 17; 8192 = 1024*8, the 1024 again 32*32).  Any other pair returns
+                             DFT3D_ERR_UNSUPPORTED.  The library chooses these too, except for axes that it runs in
+                             folded form (sums of N1 points and one product of N2, see dft3d_plan_create): 256 = 8*32
+                             on axis 0 and, with TF32 pieces, on every axis, 512 = 16*32 (not with DFT3D_SPLIT_FP16).
+                             dft3d_plan_fft_split reports the pair in use. */
   size_t workspace_limit; /* upper bound in bytes for the plan-owned workspace; 0 = default (16 GiB).  KDFT needs a
                              workspace and shrinks it to groups of n0-planes.  FFT uses one cube of workspace when it
                              fits (fewest launches), else a half, a quarter or an eighth of a cube, whichever fits

@@ -307,6 +307,12 @@ int set_kernel_attributes(int device) {
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(dft3d::fft_smem_bytes(R, NB2))))
   DFT3D_FFT_ATTR(dft3d::FFT_CONTIG, 32, 1, 16, 2, 0);
   DFT3D_FFT_ATTR(dft3d::FFT_CONTIG, 32, 2, 16, 2, 0);
+  DFT3D_FFT_ATTR(dft3d::FFT_CONTIG, 16, 1, 16, 2, 0);
+  DFT3D_FFT_ATTR(dft3d::FFT_CONTIG, 16, 2, 16, 2, 0);
+  DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 16, 1, 16, 2, 0);
+  DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 16, 2, 16, 2, 0);
+  DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 16, 1, 16, 2, 1);
+  DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 16, 2, 16, 2, 1);
   DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 32, 1, 16, 1, 0);
   DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 32, 1, 8, 2, 0);
   DFT3D_FFT_ATTR(dft3d::FFT_STRIDED, 32, 2, 8, 1, 0);
@@ -955,7 +961,9 @@ int build_fft_axis(dft3d_plan_s* p, int a, const int split[2]) {
   // of plans that leave the pieces open (512^3, microseconds per pass, this against fp16 pieces: axis 0 491 / 577,
   // axis 1 415 / 565, axis 2 394 / 428; no scaling and no larger error).  256 points (256^3: 63 / 69, 59 / 68, 63 / 59): on axis 0
   // only, since axes 1 and 2 keep the arithmetic that the launch over both of them shares.
-  if (fold_radix(n, false) && (!p->f16 || ((n == 512 || (n == 256 && a == 0)) && !(p->flags & DFT3D_SPLIT_FP16)))) {
+  // A plan that names the pair gets its two products.
+  if (fold_radix(n, false) && !split[0] && !split[1] &&
+      (!p->f16 || ((n == 512 || (n == 256 && a == 0)) && !(p->flags & DFT3D_SPLIT_FP16)))) {
     p->kax[a].n = n;
     return build_fold_axis(p, p->kax[a], fold_radix(n, false), true, scaled ? 1.0 / double(n) : 1.0);
   }
@@ -1283,7 +1291,7 @@ int fft_axis_pass(dft3d_plan_s* p, int axis, const float* in, float* out, cudaSt
     DFT3D_CUDA(cudaGetLastError());
     return DFT3D_OK;
   }
-  int nb2 = (axis == 2 || (RX == 1 && cols == 8)) ? 2 : 1;   // R = 32: the shorter lengths run folded
+  int nb2 = (axis == 2 || R == 16 || (R == 32 && RX == 1 && cols == 8)) ? 2 : 1;
   if (axis != 2 && R == 32 && RX == 1 && cols == 8) {
     // 8-line stages: two stage-2 operand buffers and one raw stage (best with direct stores), or one operand
     // buffer and two raw stages (best when the results return through the raw stage, which then stays busy longer)
@@ -1299,17 +1307,23 @@ int fft_axis_pass(dft3d_plan_s* p, int axis, const float* in, float* out, cudaSt
                                stream, map_data, ax.map_w, map_out, fp))
   if (axis == 2) {
     if (R == 32 && RX == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_CONTIG, 32, 1, 16, 2, 0); }
-    else { DFT3D_FFT_LAUNCH(dft3d::FFT_CONTIG, 32, 2, 16, 2, 0); }
+    else if (R == 32) { DFT3D_FFT_LAUNCH(dft3d::FFT_CONTIG, 32, 2, 16, 2, 0); }
+    else if (RX == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_CONTIG, 16, 1, 16, 2, 0); }
+    else { DFT3D_FFT_LAUNCH(dft3d::FFT_CONTIG, 16, 2, 16, 2, 0); }
   } else if (!stage_out) {
     if (R == 32 && RX == 1 && cols == 16) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 1, 16, 1, 0); }
     else if (R == 32 && RX == 1 && nb2 == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 1, 8, 1, 0); }
     else if (R == 32 && RX == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 1, 8, 2, 0); }
-    else { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 2, 8, 1, 0); }
+    else if (R == 32) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 2, 8, 1, 0); }
+    else if (RX == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 16, 1, 16, 2, 0); }
+    else { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 16, 2, 16, 2, 0); }
   } else {
     if (R == 32 && RX == 1 && cols == 16) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 1, 16, 1, 1); }
     else if (R == 32 && RX == 1 && nb2 == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 1, 8, 1, 1); }
     else if (R == 32 && RX == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 1, 8, 2, 1); }
-    else { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 2, 8, 1, 1); }
+    else if (R == 32) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 32, 2, 8, 1, 1); }
+    else if (RX == 1) { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 16, 1, 16, 2, 1); }
+    else { DFT3D_FFT_LAUNCH(dft3d::FFT_STRIDED, 16, 2, 16, 2, 1); }
   }
 #undef DFT3D_FFT_LAUNCH
   DFT3D_CUDA(cudaGetLastError());
@@ -1974,6 +1988,11 @@ int dft3d_plan_fft_split(dft3d_plan_t p, int axis, int* n1, int* n2) {
   if (!p || !n1 || !n2) return fail(DFT3D_ERR_INVALID_ARG, "plan, n1 and n2 must not be NULL");
   if (axis < 0 || axis > 2 || !((p->axes >> axis) & 1u) || p->amode[axis] != DFT3D_FFT)
     return fail(DFT3D_ERR_INVALID_ARG, "axis %d is not transformed in the FFT formulation by this plan", axis);
+  if (p->kax[axis].fold_r) {               // R-point sums, then one product of m points
+    *n1 = p->kax[axis].fold_r;
+    *n2 = int(p->n[axis]) / *n1;
+    return DFT3D_OK;
+  }
   *n1 = p->fax[axis].r8 ? 1024 : p->fax[axis].RX * p->fax[axis].R;
   *n2 = p->fax[axis].r8 ? 8 : p->fax[axis].R;
   return DFT3D_OK;

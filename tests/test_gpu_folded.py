@@ -298,3 +298,24 @@ def test_lines_beside_infinities_with_tf32_pieces(lib, axis):
         at[axis] = slice(None)
         lost[tuple(at)] = True
     assert not bool(torch.isfinite(z[lost]).any()) and torch.equal(z[~lost], y[~lost])
+
+
+@pytest.mark.parametrize("pieces", ["", "fp16", "tf32"])
+def test_named_pairs_are_used_and_the_query_reports_what_runs(lib, pieces):
+    """The folded form computes 256 = 8*32 and 512 = 16*32; a plan that names 16*16 or 32*16 runs those two products."""
+    from paper_2002_03260_b200 import inputs
+    shape = (256, 512, 512)
+    flags = {"": 0, "fp16": lib.DFT3D_SPLIT_FP16, "tf32": lib.DFT3D_SPLIT_TF32}[pieces]
+    x = inputs.cube(shape, "normal", 314, device="cuda")
+    want = torch.fft.fftn(x.to(torch.complex128))
+    named = [(16, 16), (32, 16), (32, 16)]
+    own = named if pieces == "fp16" else [(8, 32), (16, 32), (16, 32)]
+    for pairs in (None, named, [named[0], None, None], [None, named[1], None], [None, None, named[2]]):
+        for limit in (0, 1):
+            plan = lib.Plan(*shape, mode=lib.DFT3D_FFT, flags=flags, fft_split=pairs, workspace_limit=limit)
+            assert [plan.fft_split(a) for a in range(3)] == [(pairs or own)[a] or own[a] for a in range(3)]
+            y = plan(x)
+            torch.cuda.synchronize()
+            plan.status()
+            plan.destroy()
+            assert _rel(y, want) < BOUND
