@@ -107,8 +107,14 @@ def test_knobs_are_fixed_when_the_plan_is_created(lib, monkeypatch):
     assert (num / den) ** 0.5 < SANITY
 
 
+# the folded kernel with fp16 and TF32 pieces, the dense TF32 kernel, the real-matrix kernel in both forms, the fp16 FFT
+# kernel; contiguous and strided
 @pytest.mark.parametrize("mode_name,shape,axes", [("kdft", (64, 64, 64), None), ("kdft_tf32", (64, 64, 64), None),
-                                                 ("fft", (64, 64, 256), (2,)), ("fft", (256, 64, 64), (0,))])
+                                                 ("fft", (64, 64, 256), (2,)), ("fft", (256, 64, 64), (0,)),
+                                                 ("fft", (1024, 64, 64), (0,)), ("fft", (64, 512, 64), (1,)),
+                                                 ("fft", (64, 64, 512), (2,)),
+                                                 ("nodes", (64, 64, 64), (1,)), ("nodes", (64, 64, 64), (2,)),
+                                                 ("nodes_out", (64, 64, 64), (0,)), ("nodes_out", (64, 64, 64), (2,))])
 def test_bounded_waits_give_up_and_report(lib, oracle, monkeypatch, mode_name, shape, axes):
     """Every device-side wait has a clock budget.  Here the budget is about a millisecond and the TMA producer of every
     CTA stays silent, so nothing is ever in flight and every role's first wait runs out: the kernels return by
@@ -116,10 +122,14 @@ def test_bounded_waits_give_up_and_report(lib, oracle, monkeypatch, mode_name, s
     the oracle."""
     monkeypatch.setenv("DFT3D_TEST_SILENT_PRODUCER", "1")
     monkeypatch.setenv("DFT3D_WAIT_LIMIT_CLOCKS", "2000000")
-    mode = lib.DFT3D_FFT if mode_name == "fft" else lib.DFT3D_KDFT
-    flags = lib.DFT3D_SPLIT_TF32 if mode_name == "kdft_tf32" else 0
+    mode = lib.DFT3D_FFT if mode_name.startswith("fft") else lib.DFT3D_KDFT
+    flags = lib.DFT3D_SPLIT_TF32 if mode_name.endswith("tf32") else 0
+    flags |= lib.DFT3D_NODES_ON_OUTPUT if mode_name == "nodes_out" else 0
+    nodes = [None, None, None]
+    if mode_name.startswith("nodes"):
+        nodes[axes[0]] = _inputs().sorted_nodes(shape, 211)[axes[0]]
     x = _inputs().cube(shape, "normal", 209, device="cuda")
-    silent = lib.Plan(*shape, mode=mode, flags=flags, axes=axes)
+    silent = lib.Plan(*shape, mode=mode, flags=flags, axes=axes, nodes=nodes)
     monkeypatch.delenv("DFT3D_TEST_SILENT_PRODUCER")
     monkeypatch.delenv("DFT3D_WAIT_LIMIT_CLOCKS")
     silent(x)
@@ -128,13 +138,13 @@ def test_bounded_waits_give_up_and_report(lib, oracle, monkeypatch, mode_name, s
         silent.status()
     assert e.value.status == 5
     silent.destroy()
-    plan = lib.Plan(*shape, mode=mode, flags=flags, axes=axes)
+    plan = lib.Plan(*shape, mode=mode, flags=flags, axes=axes, nodes=nodes)
     y = plan(x)
     _finish(plan)
     plan.destroy()
     want = x.cpu().numpy().astype(np.complex128)
     for a in (axes or (0, 1, 2)):
-        want = oracle.dft_axis(want, a)
+        want = oracle.dft_axis(want, a, nodes=nodes[a], nodes_on_output=mode_name == "nodes_out")
     assert oracle.rel_l2(y.cpu().numpy(), want) < SANITY
 
 

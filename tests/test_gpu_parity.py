@@ -834,9 +834,10 @@ def test_splits_agree_512(lib, oracle):
     assert diff.item() < SANITY
 
 
+@pytest.mark.parametrize("insist", [True, False])                        # False: 512 points run the folded form with TF32 pieces
 @pytest.mark.parametrize("axis", [1, 2])
 @pytest.mark.parametrize("shape", [(64, 256, 256), (64, 512, 512)])     # 256 = 16*16; 512 = 2*16*16 (radix-2 step first)
-def test_fft_fp16_scales_every_line_on_its_own(lib, oracle, axis, shape):
+def test_fft_fp16_scales_every_line_on_its_own(lib, oracle, axis, shape, insist):
     """The fp16 split of the FFT kernel scales each line by a power of two taken from that line's largest element.
     Lines that differ by up to 2^120 in magnitude must each come out with fp32-level error relative to their OWN norm
     (a single scale for the whole array would flush the small lines to zero)."""
@@ -846,7 +847,7 @@ def test_fft_fp16_scales_every_line_on_its_own(lib, oracle, axis, shape):
     expo = torch.randint(-60, 61, [shape[d] for d in other], generator=g, device="cuda").to(torch.float32)
     scale = torch.exp2(expo).unsqueeze(axis)
     xs = (x * scale).contiguous()
-    plan = lib.Plan(*shape, mode=lib.DFT3D_FFT, flags=lib.DFT3D_SPLIT_FP16, axes=(axis,))
+    plan = lib.Plan(*shape, mode=lib.DFT3D_FFT, flags=lib.DFT3D_SPLIT_FP16 if insist else 0, axes=(axis,))
     ys = plan(xs)
     _finish(plan)
     plan.destroy()
@@ -879,28 +880,28 @@ def test_destroy_input_uses_the_input_as_workspace(lib, oracle, mode_name, shape
 
 
 def test_kdft_cta_pair_kernel_matches(lib, oracle, monkeypatch):
-    """The cta_group::2 form of the fp16 KDFT kernel (pairs of CTAs share every table tile; enabled with
-    DFT3D_KDFT_PAIR=1 at plan creation) computes the same sums in the same order: identical bits, and a ragged
-    shape against the oracle."""
-    shape = (256, 128, 384)
-    x = _inputs().cube(shape, "normal", 99, device="cuda")
-    plan = lib.Plan(*shape, flags=lib.DFT3D_SPLIT_FP16)
-    want = plan(x)
-    _finish(plan)
-    plan.destroy()
-    monkeypatch.setenv("DFT3D_KDFT_PAIR", "1")
-    plan = lib.Plan(*shape, flags=lib.DFT3D_SPLIT_FP16)
-    got = plan(x)
-    _finish(plan)
-    plan.destroy()
-    assert torch.equal(got, want)
-    shape = (132, 260, 200)
-    x = _inputs().cube(shape, "normal", 100, device="cuda")
-    plan = lib.Plan(*shape, flags=lib.DFT3D_SPLIT_FP16)
-    y = plan(x)
-    _finish(plan)
-    plan.destroy()
-    assert oracle.rel_l2(y.cpu().numpy(), oracle.dft3d(x.cpu().numpy())) < SANITY
+    """The cta_group::2 form of the fp16 KDFT kernel (pairs of CTAs share every table tile; the default from 2048 points,
+    from 128 points with DFT3D_KDFT_PAIR=1 at plan creation) on the complex matrix, against the real-matrix form of
+    the same product and the oracle.  Uniform axes with a folded form never run it, so the axes have nodes; the second
+    shape has ragged tiles, and the uniform 260 points of the third have no folded form."""
+    for shape, uniform in (((256, 128, 384), False), ((132, 260, 200), False), ((12, 260, 8), True)):
+        x = _inputs().cube(shape, "normal", 99, device="cuda")
+        nodes = None if uniform else _inputs().sorted_nodes(shape, 100)
+        axes = (1,) if uniform else None
+        got = []
+        for pair in ("0", "1"):
+            monkeypatch.setenv("DFT3D_KDFT_PAIR", pair)
+            plan = lib.Plan(*shape, flags=lib.DFT3D_SPLIT_FP16, nodes=nodes, axes=axes)
+            got.append(plan(x))
+            _finish(plan)
+            plan.destroy()
+        assert not torch.equal(got[0], got[1])          # two kernels
+        assert _rel_l2_gpu(got[1], got[0]) < SANITY
+        if uniform:
+            want = oracle.dft_axis(x.cpu().numpy().astype(np.complex128), 1)
+        else:
+            want = oracle.dft3d(x.cpu().numpy(), nodes=nodes)
+        assert oracle.rel_l2(got[1].cpu().numpy(), want) < SANITY
 
 
 # ------------------------------------------------------------------ the largest supported length

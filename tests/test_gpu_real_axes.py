@@ -32,18 +32,24 @@ def test_nodes_on_single_axes(lib, oracle, shape, axes, on_output, sign):
     full = inputs.sorted_nodes(shape, 402)
     nodes = [full[a] * 3.0 - 1.0 if a in axes else None for a in range(3)]     # any finite value, used modulo 1
     flags = lib.DFT3D_NODES_ON_OUTPUT if on_output else 0
-    guard = torch.full((1 << 14,), 7.0, device="cuda")
     plan = lib.Plan(*shape, nodes=nodes, axes=axes, sign=sign, flags=flags)
-    y = plan(x)
+    # input and output (all NaN before) between margins that must not change
+    margin = 1 << 12
+    bufs = [torch.full((x.numel() + 2 * margin,), 7.0 + 7.0j, dtype=torch.complex64, device="cuda") for _ in range(2)]
+    xi, y = [b[margin:margin + x.numel()].view(shape) for b in bufs]
+    xi.copy_(x)
+    y.fill_(complex(float("nan"), float("nan")))
+    plan(xi, y)
     torch.cuda.synchronize()
     plan.status()
     plan.destroy()
+    assert all(bool((b[:margin] == 7.0 + 7.0j).all()) and bool((b[-margin:] == 7.0 + 7.0j).all()) for b in bufs)
+    assert torch.equal(xi, x)
     want = x.cpu().numpy().astype(np.complex128)
     for a in axes:
         want = oracle.dft_axis(want, a, sign=sign, scale=1.0 / shape[a] if sign > 0 else 1.0, nodes=nodes[a],
                                nodes_on_output=on_output)
     assert oracle.rel_l2(y.cpu().numpy(), want) < 5e-6
-    assert bool((guard == 7.0).all())
 
 
 @pytest.mark.parametrize("on_output", [False, True])
