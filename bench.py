@@ -64,6 +64,21 @@ def conv_flops(n):
     return 5.0 * P * math.log2(P)
 
 
+def kdft_axis_form(n, with_nodes, f16):
+    """(kernel, tensor flops issued per point) of a KDFT axis of n points: three split products of the complex matrix (8 n
+    flops per point), of a real matrix on both parts (4 n), or of the m-point matrix that the residue classes of a
+    folded axis share (8 m); csrc/dft3d_api.cu has the rule."""
+    if not with_nodes:
+        radices = (4, 8, 16) if n % 4 == 0 or f16 else (1, 2, 3, 5, 6, 10)
+        for r in radices:
+            if n % r == 0 and n // r <= (64 if f16 else 32):
+                return "fold_axis_kernel", 24.0 * (n // r)
+    if not f16:
+        return "kdft_axis_kernel", 24.0 * n
+    paired = n >= 2048 if "DFT3D_KDFT_PAIR" not in os.environ else (os.environ["DFT3D_KDFT_PAIR"] != "0" and n >= 128)
+    return ("kdft_f16x2_axis_kernel", 24.0 * n) if paired else ("kdft_real_axis_kernel", 12.0 * n)
+
+
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_bytes_per_point.json")
 
 
@@ -311,14 +326,19 @@ def run_configs(args):
             f16 = plan.split == dft.DFT3D_SPLIT_FP16
             if mode == "kdft":
                 gemm = 8.0 * sum(shape) * P
-                issued = 3.0 * gemm
+                forms = [kdft_axis_form(v, with_nodes, f16) for v in shape]
+                issued = sum(f for _, f in forms) * P
                 peak = peaks["bf16_tflops_sustained"] * (1.0 if f16 else 1.1 / 2.25)
-                roof = {"bound": "tensor", "achieved": issued / (med * 1e-3) * 1e-12, "peak": peak, "unit": "TFLOP/s",
-                        "peak_source": "%s bf16 sustained%s" % (peak_kind, "" if f16 else " x 1.1/2.25 (TF32)")}
+                if all(k == "fold_axis_kernel" for k, _ in forms):
+                    roof = {"bound": "hbm", "achieved": 48.0 * P / (med * 1e-3) * 1e-9, "peak": peaks["hbm_gbs"],
+                            "unit": "GB/s", "peak_source": "%s STREAM-style copy" % peak_kind}
+                else:
+                    roof = {"bound": "tensor", "achieved": issued / (med * 1e-3) * 1e-12, "peak": peak, "unit": "TFLOP/s",
+                            "peak_source": "%s bf16 sustained%s" % (peak_kind, "" if f16 else " x 1.1/2.25 (TF32)")}
             else:
                 splits = [plan.fft_split(a) for a in range(3)]
                 gemm = 8.0 * sum(a + b for a, b in splits) * P
-                issued = 3.0 * 8.0 * sum(2 * b for a, b in splits) * P
+                issued = 3.0 * 8.0 * sum(b if a < b else 2 * b for a, b in splits) * P     # N1 < N2: folded, one product
                 roof = {"bound": "hbm", "achieved": 48.0 * P / (med * 1e-3) * 1e-9, "peak": peaks["hbm_gbs"],
                         "unit": "GB/s", "peak_source": "%s STREAM-style copy" % peak_kind}
             roof["frac"] = roof["achieved"] / roof["peak"]
@@ -483,16 +503,17 @@ def main():
             algo_flops = 8.0 * nsum * P
             issued = 3.0 * algo_flops
             ach = issued / (ms * 1e-3) * 1e-12
-            if split == dft.DFT3D_SPLIT_FP16 and all(any(shape[a] % r == 0 and shape[a] // r <= 64 for r in (4, 8, 16)) for a in taxes):
+            forms = [kdft_axis_form(shape[a], False, split == dft.DFT3D_SPLIT_FP16)[0] for a in taxes]
+            if all(f == "fold_axis_kernel" for f in forms):
                 # every axis in folded form (csrc/fold_kernel.cuh): one pass over the cube per axis, bound by HBM
                 moved = len(taxes) * 16.0 * P
                 return {"bound": "hbm", "kernel": "fold_axis_kernel", "achieved": moved / (ms * 1e-3) * 1e-9,
                         "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": moved / (ms * 1e-3) * 1e-9 / peaks["hbm_gbs"],
                         "traffic": (dram_bytes_per_point("fold_axis_kernel")[0] or 0.0) * P or None,
-                        "peak_source": "%s STREAM-style copy" % peak_kind, "avg_launch_ms": ms / (nlaunch - 1),
+                        "peak_source": "%s STREAM-style copy" % peak_kind, "avg_launch_ms": ms / len(taxes),
                         "bytes": "8 B read + 8 B written per point per axis pass (the reduction over the input comes on top)"}
             if split == dft.DFT3D_SPLIT_FP16:
-                paired = max(shape[a] for a in taxes) >= 2048 and os.environ.get("DFT3D_KDFT_PAIR", "1") != "0"
+                paired = "kdft_f16x2_axis_kernel" in forms
                 kernel = "kdft_f16x2_axis_kernel" if paired else "kdft_real_axis_kernel"   # CTA pairs from 2048 points up
                 if not paired:                      # a real matrix on real and imaginary parts: half the multiplications
                     algo_flops *= 0.5
@@ -517,10 +538,12 @@ def main():
         if mode == "kdft":
             roofline = kdft_roofline(ms_step, launches, psplit)
         else:
-            # only kernel: fft_axis_kernel, one launch per axis; algorithmic traffic 16 B per point per axis
+            # one launch per axis; algorithmic traffic 16 B per point per axis
             algo_bytes = len(taxes) * 16.0 * P
             achieved = algo_bytes / (ms_step * 1e-3) * 1e-9
             fkernel = "fft_f16_axis_kernel" if psplit == dft.DFT3D_SPLIT_FP16 else "fft_axis_kernel"
+            if all(shape[a] == 512 or (shape[a] == 256 and psplit == dft.DFT3D_SPLIT_TF32) for a in taxes) and args.split != "fp16":
+                fkernel = "fold_axis_kernel"
             roofline = {"bound": "hbm", "kernel": fkernel, "achieved": achieved, "peak": peaks["hbm_gbs"],
                         "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"],
                         "traffic": (dram_bytes_per_point(fkernel)[0] or 0.0) * P or None,

@@ -54,7 +54,8 @@ enum {
      pieces whose products are accumulated).  Both use 3
      products of 11-bit pieces with fp32 accumulation and meet the same error bound.  Default: fp16 pieces (KDFT:
      when every transformed n_a % 4 == 0, TF32 pieces otherwise); FFT axes of 512 points and axes 0 of 256 points
-     take TF32 pieces unless fp16 ones are insisted on. */
+     take TF32 pieces unless fp16 ones are insisted on or the factor pair is named.  Either way a line comes out with
+     its precision at any magnitude: fp16 FFT pieces are scaled line by line, TF32 ones near the ends of the range. */
   DFT3D_SPLIT_FP16 = 4u,        /* insist on fp16 pieces (operands scaled by exact powers of two: KDFT from the largest
                                    input magnitude, FFT per line; half the tensor-core instructions of TF32);
                                    DFT3D_ERR_UNSUPPORTED for KDFT when a transformed n_a is not a multiple of 4 */

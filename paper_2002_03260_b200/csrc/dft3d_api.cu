@@ -630,8 +630,7 @@ cudaError_t launch_overlapped(const dft3d_plan_s* p, void (*kernel)(Params...), 
 }
 
 // One KDFT axis pass over a [batches][J][C] complex view (STRIDED) or rows x J (CONTIG).
-template <class Params>
-void fill_f16_params(Params& fp, const dft3d::KdftParams& kp, const KdftAxis& ax, dft3d_plan_s* p, int chain_pos) {
+void fill_f16_params(dft3d::KdftF16Params& fp, const dft3d::KdftParams& kp, const KdftAxis& ax, dft3d_plan_s* p, int chain_pos) {
   fp.k2 = kp.k2; fp.bn = kp.bn; fp.n_tiles = kp.n_tiles; fp.chunk_kb = kp.chunk_kb;
   fp.m_tiles = kp.m_tiles; fp.rows = kp.rows; fp.batches = kp.batches; fp.C = kp.C;
   fp.lpb = kp.lpb; fp.bpt = kp.bpt; fp.c_tiles = kp.c_tiles;
@@ -642,7 +641,7 @@ void fill_f16_params(Params& fp, const dft3d::KdftParams& kp, const KdftAxis& ax
   fp.wc = kp.wc;
   // paired-CTA kernel: eight table panels live at a time once there are sixteen or more (measured: 8192 x 8192 26.9 -> 24.5 ms,
   // 64 x 4096 x 4096 214 -> 202 ms, 2048^3 unchanged; groups of 1, 2, 4, 16, 32 panels are slower)
-  fp.n_group = p->knobs.kdft_ngroup >= 0 ? p->knobs.kdft_ngroup : ((kp.n_tiles >= 16 && ax.pair) ? 8 : 0);
+  fp.n_group = p->knobs.kdft_ngroup >= 0 ? p->knobs.kdft_ngroup : (kp.n_tiles >= 16 ? 8 : 0);
 }
 
 // One pass in the real form; the lines of axis 2 are `batches` rows, those of axes 0 and 1 the columns of a
@@ -958,8 +957,8 @@ int build_fft_axis(dft3d_plan_s* p, int a, const int split[2]) {
   ax.cols = (R == 32 && RX == 4) ? 4 : ((R == 32 && RX == 2) ? 8 : 16);   // a 128 KB stage holds all n rows of `cols` lines
                                                                            // (fft_axis_pass may pick 8 for R = 32, RX = 1)
   // One product in folded form, with TF32 pieces, instead of two: always where the plan has TF32 pieces, and on 512-point axes
-  // of plans that leave the pieces open (512^3, microseconds per pass, this against fp16 pieces: axis 0 491 / 577,
-  // axis 1 415 / 565, axis 2 394 / 428; no scaling and no larger error).  256 points (256^3: 63 / 69, 59 / 68, 63 / 59): on axis 0
+  // of plans that leave the pieces open (512^3, microseconds per pass, this against fp16 pieces: axis 0 479 / 574,
+  // axis 1 444 / 564, axis 2 416 / 441; no larger error).  256 points (256^3: 56 / 72, 59 / 68, 63 / 59): on axis 0
   // only, since axes 1 and 2 keep the arithmetic that the launch over both of them shares.
   // A plan that names the pair gets its two products.
   if (fold_radix(n, false) && !split[0] && !split[1] &&
@@ -1167,7 +1166,7 @@ int fft_axis_pass(dft3d_plan_s* p, int axis, const float* in, float* out, cudaSt
       // prefetching helps while rows are close (axis 1); with rows MiBs apart (axis 0) the pass is bound by the
       // rate of address translations and every extra request costs more than it hides (measured: 10.0 -> 12.2 ms)
       // The fp16 kernel with R = 32 keeps up without (axis 1 of 100 x 1024 x 1024: 370 us without, 377 us with; 60 x 2048 x 1024
-      // 536 / 541; 8192 x 8192 914 / 933).
+      // 536 / 541).
       fp.l2_prefetch = kn.fft_l2_prefetch >= 0 ? kn.fft_l2_prefetch : (C * 8 < (1ll << 20) && !(p->f16 && R == 32) ? 1 : 0);
       if (n2_sub) fp.l2_prefetch = 0;
     }

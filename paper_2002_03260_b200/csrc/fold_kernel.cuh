@@ -10,16 +10,17 @@
 //
 // Pieces: x = hi + 2^-11 * lo', W likewise, hi and lo' in fp16 (11-bit significands); hi x [W_hi | W_lo'] is one MMA of
 // twice the width, lo' x W_hi is added to its upper half, and the store forms hi*hi + 2^-11 * cross in fp32.  Because
-// the lo pieces carry their own 2^11 they stay normal numbers: an element keeps its 22 bits down to 2^-25 of the largest
-// one and the absolute error never exceeds about 2^-46 of it.  The chains on the large accumulator are 2m/16 <= 8
-// MMAs long.  Scales are exact powers of two (table 1024 * W, data from the largest input magnitude).
+// the lo pieces carry their own 2^11 they stay normal numbers: an element is held to 2^-23 of itself down to 2^-25 of the
+// largest one and to about 2^-46 of that one below; the R-point sums and the phases round in fp32 on top.  The chains on the
+// large accumulator are 2m/16 <= 8 MMAs long.  Scales are exact powers of two (table 1024 * W, data from the largest input
+// magnitude; TF32 pieces: see FoldRange).
 //
 // Roofline: HBM, 16 B per point.  Per tile of 128 lanes (128/R lines x R classes) and m = 64: 24 MMAs = 1536 clk of the
 // tensor pipe and about 2600 clk of shared-memory traffic against 5700 clk of an SM's share of the HBM stream.
 //
-// Measured (per transform, the reduction over the input included): 512^3 5.14 -> 1.44 ms, 1024^3 74.8 -> 13.3 ms, 64^3
-// 38.9 -> 27.7 us against the full matrix; a contiguous 1024-point pass moves 5.9 TB/s, a strided one 4.2-4.6 TB/s.  Relative
-// error against 64-bit results 2e-7 to 5e-7 per 3D transform (full matrix: 1.5e-6 to 2.6e-6).
+// Measured (per transform, the reduction over the input included; overlapped launches): 512^3 4.7 -> 1.48-1.6 ms, 1024^3 75
+// -> 13.1 ms, 64^3 38 -> 19.1 us against the full matrix; a contiguous 1024-point pass moves 5.8 TB/s, a strided one 4.2-4.6
+// TB/s.  Relative error against 64-bit results 2e-7 to 5e-7 per 3D transform (full matrix: 1.5e-6 to 2.6e-6).
 //
 // Organisation (one persistent CTA per SM, 640 threads):
 //   warp 0       table load; one thread issues tcgen05.mma (both operands from shared memory)
@@ -27,7 +28,7 @@
 //   warps 8-19   global -> registers -> R-point sums, phase, split -> shared memory; L2 prefetch two tiles ahead
 // Two operand buffers and two accumulators, so the three run on different tiles.  No TMA on the data: the loads are
 // coalesced as they are (16 or more neighbouring columns, or consecutive points of a line) and need no alignment beyond
-// a complex number's 8 bytes.
+// a complex number's 8 bytes (contiguous lines of even m: 16 bytes, which every plan asks of its arrays).
 #pragma once
 #include <type_traits>
 #include "kdft_f16_kernel.cuh"

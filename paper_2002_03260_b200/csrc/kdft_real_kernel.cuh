@@ -17,8 +17,9 @@
 // contraction) arrives as halves with a barrier pair of their own.
 //
 // Bound: the instructions of the split and epilogue warps (tensor pipe a third busy at 256 points).  Nodes on all axes of 256^3,
-// the reduction included: 414 us with the complex matrix, 245 us in this form (a pass 100 to 127 -> 68 us).  Two table stages
-// and five half stages of raw data against three and two: 281 and 287 us before the epilogue was shortened.
+// the reduction included: 405-414 us with the complex matrix; in this form 246 us back to back on one input and 271 us on
+// changing inputs (nodes on the output 259 us); a pass 100 to 127 -> 68 us.  Two table stages and five half stages of raw data
+// against three and two: 281 and 287 us before the epilogue was shortened.
 #pragma once
 #include "kdft_f16_kernel.cuh"
 
