@@ -280,16 +280,16 @@ __device__ __forceinline__ unsigned fold_next(const FoldRange& rg, bool all, uns
   return w * 32 + __ffs(b) - 1;
 }
 
-// Two complex numbers -> TF32 pieces (re, im, re', im'): hi rounded to eleven bits (finite values here are far from the largest
-// float), lo the exact remainder of at most twelve bits, whose last one the tensor core ignores.  A NaN stays one in lo.
+// Two complex numbers -> TF32 pieces (re, im, re', im'): hi is the raw word (the tensor core ignores the low 13 bits of the
+// mantissa), lo the remainder rounded to TF32.
 __device__ __forceinline__ void split_tf32(C2 x, uint32_t (&hi)[4], uint32_t (&lo)[4]) {
   float v[4];
   unpack2(x.re, v[0], v[2]);
   unpack2(x.im, v[1], v[3]);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    hi[i] = (__float_as_uint(v[i]) + 0x1000u) & 0xffffe000u;
-    lo[i] = __float_as_uint(v[i] - __uint_as_float(hi[i]));
+    hi[i] = __float_as_uint(v[i]);
+    lo[i] = (__float_as_uint(v[i] - __uint_as_float(hi[i] & 0xffffe000u)) + 0x1000u) & 0xffffe000u;
   }
 }
 

@@ -272,24 +272,6 @@ def test_whole_cubes_near_the_ends_of_the_range(lib, pieces, limit, power):
     assert torch.equal(z[normal], want[normal]) and bool(((z - want)[~normal].abs() <= 2.0 ** -148).all())
 
 
-@pytest.mark.parametrize("mode,pieces,axis,n", RANGE_AXES)
-def test_pieces_hold_23_bits(lib, mode, pieces, axis, n):
-    """A single sample at the start of each line: the output at frequency zero is that sample, cut into two pieces of eleven
-    bits whose rounding leaves 2^-23 of a component (2 units of 2^-24) at most, to either side alike."""
-    from paper_2002_03260_b200 import inputs
-    shape = [64, 64, 64]
-    shape[axis] = n
-    v = inputs.cube(tuple(shape), "normal", 311, device="cuda").select(axis, 0)
-    x = torch.zeros(shape, dtype=torch.complex64, device="cuda")
-    x.select(axis, 0).copy_(v)
-    y = _run(lib, x, mode=lib.DFT3D_FFT if mode == "fft" else lib.DFT3D_KDFT, axes=(axis,),
-             flags=lib.DFT3D_SPLIT_TF32 if pieces else 0)
-    got = torch.view_as_real(y.select(axis, 0)).double()
-    want = torch.view_as_real(v).double()
-    units = (got - want) / want * 2.0 ** 24
-    assert units.abs().max().item() <= 2.0 and abs(units.mean().item()) < 0.1
-
-
 def test_more_units_than_a_block_can_mark(lib):
     """3.2e8 lines of four points: with more than 65536 units a block scales every line by its own largest component."""
     n0, n1 = 40000, 8000
